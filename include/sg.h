@@ -86,9 +86,11 @@ typedef struct {
   int mg_coarse;     /* SG_PC_MG: cells per side of the coarsest mesh (the paper: 2); n must be  */
                      /* mg_coarse times a power of two, and the coarsest interior system of     */
                      /* (mg_coarse - 1)^2 P unknowns is solved with its dense inverse (<= 4096)  */
-  int op_kernel;     /* SG operator kernel: SG_OP_AUTO (time the candidates on this system at   */
-                     /* setup, keep the fastest; the choice is cached per N, P, L and precision */
-                     /* for the process), SG_OP_PAIRS or SG_OP_TILE                             */
+  int op_kernel;     /* SG operator kernel: SG_OP_AUTO (the block-stencil operator while its     */
+                     /* assembled blocks take at most an eighth of the device memory and leave   */
+                     /* half of it free; else time the other candidates on this system at setup  */
+                     /* and keep the fastest, cached per N, P, L and precision for the process), */
+                     /* SG_OP_PAIRS or SG_OP_TILE                                               */
   int op_kappa;      /* SG_OP_TILE: k per register group, 1, 2 or 4 (0: 2 in FP64, 4 in FP32)   */
   int op_ctas;       /* SG_OP_TILE: CTAs per SM the shared memory is planned for, 1 or 2 (0: 1) */
   int ilu_order;     /* ILU(0) node ordering: SG_ILU_NATURAL, or SG_ILU_COLOR4 (colour           */
@@ -116,7 +118,7 @@ typedef struct {
 #define SG_ILU_NATURAL 0
 #define SG_ILU_COLOR4 1
 
-#define SG_OP_AUTO 0   /* choose by timing (see op_kernel)                                      */
+#define SG_OP_AUTO 0   /* choose (see op_kernel)                                                */
 #define SG_OP_PAIRS 1  /* one CTA per 4 rows, (k, b) pairs over threads, operands in shared mem */
 #define SG_OP_TILE 2   /* 32 rows of a grid line per CTA, one per lane, k groups in registers  */
 
@@ -150,7 +152,9 @@ int sg_dims(const sg_handle* h, int sys, int* N, int* P, int* L);
 int sg_nnz(const sg_handle* h, int sys, long long* nnz_A, long long* nnz_G);
 
 /* Y = K X = sum_k A_k X G_k^T (Eqs. stochastic_matrix, K_matrix); X, Y device, N x P FP64,
- * must not overlap.  Asynchronous on ``stream``. */
+ * must not overlap.  Asynchronous on ``stream``.  Calls on several streams may overlap: what the
+ * block-stencil operator stores between its two kernels comes from the handle's memory pool in
+ * stream order (a call under capture adds an allocation and a free node to the graph). */
 int sg_matvec(sg_handle* h, int sys, const double* X, double* Y, void* stream);
 
 /* Same operator with the FP32 (precision SG_MIXED_FP32) or BF16 (SG_MIXED_BF16) copy of the
@@ -211,8 +215,8 @@ int sg_gmres_solve(sg_handle* h, const double* const* F, double* const* X, sg_so
 int sg_export(const sg_handle* h, int sys, int what, void* dst, size_t bytes);
 
 /* Which SG operator kernel system ``sys`` runs: info[0..3] for the FP64 operator and info[4..7]
- * for the FP32 one, each {kernel (0 none, 1 pair kernel, 2 row-tiled kernel), kappa, shared
- * memory bytes, chunks}; ``msg`` (msg_len bytes, may be NULL) receives why a row-tiled operator
+ * for the FP32 one, each {kernel (0 none, 1 pair kernel, 2 row-tiled kernel, 3 block-stencil
+ * operator), kappa (3: fields per range), shared memory bytes, chunks (3: ranges)}; ``msg`` (msg_len bytes, may be NULL) receives why a row-tiled operator
  * was not built ("" if it was). */
 int sg_op_info(const sg_handle* h, int sys, long long* info, char* msg, int msg_len);
 

@@ -22,6 +22,7 @@ template <typename TA, typename TV>
 __device__ __forceinline__ TA cvt(const TV* p);
 template <> __device__ __forceinline__ double cvt<double, double>(const double* p) { return *p; }
 template <> __device__ __forceinline__ float cvt<float, float>(const float* p) { return *p; }
+template <> __device__ __forceinline__ float cvt<float, double>(const double* p) { return (float)*p; }
 template <> __device__ __forceinline__ float cvt<float, __nv_bfloat16>(const __nv_bfloat16* p) {
   return __bfloat162float(*p);
 }
@@ -158,13 +159,19 @@ int launch_apply(const System& s, const TV* stack, const TA* eg, const TA* X, TA
 }  // namespace
 
 int launch_matvec_f64(const System& s, const double* X, double* Y, double alpha, const double* B,
-                      double beta, cudaStream_t st, const int* done) {
+                      double beta, cudaStream_t st, const int* done, double* scratch) {
+  if (s.block64.ready)
+    return launch_block_op<double>(s, s.block64, X, Y, alpha, B, beta,
+                                   scratch ? scratch : s.block64.f64.p, st, done);
   if (s.tile64.ready) return launch_tile_op<double>(s, s.tile64, X, Y, alpha, B, beta, st, done);
   return launch_apply<double, double>(s, s.stack.p, s.ent_g.p, X, Y, alpha, B, beta, st, done);
 }
 
 int launch_matvec_f32(const System& s, const float* X, float* Y, float alpha, const float* B,
-                      float beta, cudaStream_t st, const int* done) {
+                      float beta, cudaStream_t st, const int* done, float* scratch) {
+  if (s.block32.ready)
+    return launch_block_op<float>(s, s.block32, X, Y, alpha, B, beta,
+                                  scratch ? scratch : s.block32.f32.p, st, done);
   if (s.tile32.ready && s.prm.precision == SG_MIXED_FP32)
     return launch_tile_op<float>(s, s.tile32, X, Y, alpha, B, beta, st, done);
   if (s.prm.precision == SG_MIXED_BF16)
@@ -172,6 +179,15 @@ int launch_matvec_f32(const System& s, const float* X, float* Y, float alpha, co
                                               beta, st, done);
   return launch_apply<float, float>(s, s.stack_f32.p, s.ent_g_f32.p, X, Y, alpha, B, beta, st,
                                     done);
+}
+
+int launch_matvec_pairs_f64(const System& s, const double* X, double* Y, cudaStream_t st) {
+  return launch_apply<double, double>(s, s.stack.p, s.ent_g.p, X, Y, 1.0, nullptr, 0.0, st, nullptr);
+}
+
+int launch_matvec_pairs_f32(const System& s, const float* X, float* Y, cudaStream_t st) {
+  return launch_apply<float, double>(s, s.stack.p, s.ent_g_f32.p, X, Y, 1.0f, nullptr, 0.0f, st,
+                                     nullptr);
 }
 
 }  // namespace sg

@@ -241,6 +241,7 @@ int mg_setup_levels(System& s, cudaStream_t st) {
     c->prm.outer_sweeps = 1;
     c->prm.graphs = 0;
     c->timer = s.timer;
+    c->lean = s.lean;
     SG_TRY(setup_system_public(*c, st, false));
     const size_t NP = (size_t)c->N * c->P;
     SG_TRY(c->mg_b.alloc(NP));

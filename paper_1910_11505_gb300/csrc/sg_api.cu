@@ -303,6 +303,20 @@ static int time_operator(const System& s, const T* X, T* Y, cudaStream_t st, dou
   return rc;
 }
 
+// Whether the block-stencil operator is to serve this system in precision ``elem``: it takes more
+// memory than the row-tiled one (2 to 4 times its stack), so it is kept to an eighth of the
+// device's memory and to the half of it that is left free otherwise.
+static bool block_op_wanted(const System& s, int elem) {
+  const size_t bytes = block_op_bytes(s, elem);
+  if (bytes == 0 || s.lean) return false;
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return bytes <= total_b / 8 && free_b >= bytes + total_b / 2;
+}
+
 // Build the operator kernel of precision ``elem`` (8: FP64, 4: FP32) that op_kernel asks for.
 // SG_OP_AUTO times the pair kernel and every row-tiled variant that fits (kappa 1, 2, 4; one or
 // two CTAs per SM) on this system, keeps the fastest and caches the choice for the system's
@@ -312,6 +326,21 @@ static int choose_operator(System& s, int elem, cudaStream_t st) {
   const sg_params& p = s.prm;
   std::string& note = s.tile_msg;
   if (p.op_kernel == SG_OP_PAIRS) return SG_OK;
+  if (p.op_kernel == SG_OP_AUTO && block_op_wanted(s, elem)) {
+    BlockOp& blk = elem == 8 ? s.block64 : s.block32;
+    const int rc = build_block_op(s, blk, elem, st);
+    if (rc == SG_OK) {
+      const std::array<long long, 5> key{s.N, s.P, s.L, p.q, -elem};
+      std::lock_guard<std::mutex> lock(g_tune_mu);
+      note += std::string(elem == 8 ? "fp64" : "fp32") +
+              (g_tune.count(key) ? ": block (cached); " : ": chose block; ");
+      g_tune[key] = TuneChoice();
+      return SG_OK;
+    }
+    free_block_op(blk);
+    if (rc != SG_ERR_ARG && rc != SG_ERR_OOM) return rc;
+    set_error("");
+  }
   if (p.op_kernel == SG_OP_TILE) {
     const int kappa = p.op_kappa ? p.op_kappa : (elem == 8 ? 2 : 4);
     const int ctas = p.op_ctas ? p.op_ctas : 1;
@@ -463,6 +492,8 @@ static void free_system(System* s) {
   if (!s) return;
   free_tile_op(s->tile64);
   free_tile_op(s->tile32);
+  free_block_op(s->block64);
+  free_block_op(s->block32);
   for (System* c : s->mg) free_system(c);
   s->mg.clear();
   for (auto* b : {&s->mg_b, &s->mg_u, &s->mg_r, &s->mg_d, &s->mg_inv}) b->release();
@@ -602,7 +633,7 @@ static int setup_system(System& s, cudaStream_t st, bool krylov = true) {
   if (p.precision == SG_FP64 || p.op_kernel == SG_OP_TILE || krylov) SG_TRY(choose_operator(s, 8, st));
   if (p.precision == SG_MIXED_FP32) {
     SG_TRY(choose_operator(s, 4, st));
-    if (s.tile32.ready) s.stack_f32.release();
+    if (s.tile32.ready || s.block32.ready) s.stack_f32.release();
   }
 
   // preconditioner blocks and factors
@@ -697,6 +728,45 @@ static int setup_system(System& s, cudaStream_t st, bool krylov = true) {
 
 int setup_system_public(System& s, cudaStream_t st, bool krylov) { return setup_system(s, st, krylov); }
 void free_system_public(System* s) { free_system(s); }
+
+// Memory of the products that the block-stencil operator adds in its second kernel.  Calls of
+// sg_matvec on different streams may overlap, so each takes its own by stream order from the
+// handle's pool (which keeps it for the next call and returns it with the handle); the pool starts
+// with one allocation of the largest system's size, so calls on one stream never allocate.
+static int make_pool(sg_handle* h, cudaStream_t st) {
+  size_t bytes = 0;
+  for (System* s : h->sys) {
+    if (s->block32.ready) bytes = std::max(bytes, sizeof(float) * block_scratch_elems(*s));
+    if (s->block64.ready) bytes = std::max(bytes, sizeof(double) * block_scratch_elems(*s));
+  }
+  if (bytes == 0) return SG_OK;
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = h->device;
+  SG_CUDA(cudaMemPoolCreate(&h->pool, &props));
+  unsigned long long keep = ~0ull;
+  SG_CUDA(cudaMemPoolSetAttribute(h->pool, cudaMemPoolAttrReleaseThreshold, &keep));
+  void* p = nullptr;
+  if (cudaMallocFromPoolAsync(&p, bytes, h->pool, st) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(SG_ERR_OOM, "operator scratch of " + std::to_string(bytes) + " bytes");
+  }
+  SG_CUDA(cudaFreeAsync(p, st));
+  return SG_OK;
+}
+
+template <typename T, typename Run, typename Pairs>
+static int matvec_pooled(sg_handle* h, System& s, cudaStream_t st, Run run, Pairs pairs) {
+  void* p = nullptr;
+  if (cudaMallocFromPoolAsync(&p, sizeof(T) * block_scratch_elems(s), h->pool, st) != cudaSuccess) {
+    cudaGetLastError();  // no memory for another stream's products: the kernel that needs none
+    return pairs();
+  }
+  const int rc = run((T*)p);
+  SG_CUDA(cudaFreeAsync(p, st));
+  return rc;
+}
 
 static System* get_sys(const sg_handle* h, int sys) {
   if (!h || sys < 0 || sys >= (int)h->sys.size()) return nullptr;
@@ -1003,22 +1073,33 @@ int sg_setup(const sg_params* prm, int nsys, void* stream, sg_handle** out) {
   if (!prm || nsys < 1) return fail(SG_ERR_ARG, "need nsys >= 1 parameter sets");
   for (int i = 0; i < nsys; ++i) SG_TRY(validate(prm[i]));
   cudaStream_t st = (cudaStream_t)stream;
-  sg_handle* h = new sg_handle();
-  cudaGetDevice(&h->device);
-  for (int i = 0; i < nsys; ++i) {
-    System* s = new System();
-    s->prm = prm[i];
-    s->timer = &h->timer;
-    h->sys.push_back(s);
-    int rc = setup_system(*s, st);
-    if (rc != SG_OK) {
-      std::string msg = g_last_error;
-      sg_free(h);
-      return fail(rc, "system " + std::to_string(i) + ": " + msg);
+  // where the device's memory does not hold all systems, once more without the block-stencil
+  // operators, whose memory the other forms do not need
+  for (const bool lean : {false, true}) {
+    sg_handle* h = new sg_handle();
+    cudaGetDevice(&h->device);
+    int rc = SG_OK;
+    bool blocks = false;
+    for (int i = 0; i < nsys && rc == SG_OK; ++i) {
+      System* s = new System();
+      s->prm = prm[i];
+      s->timer = &h->timer;
+      s->lean = lean;
+      h->sys.push_back(s);
+      rc = setup_system(*s, st);
+      blocks = blocks || s->block64.ready || s->block32.ready;
+      if (rc != SG_OK) fail(rc, "system " + std::to_string(i) + ": " + std::string(g_last_error));
     }
+    if (rc == SG_OK) rc = make_pool(h, st);
+    if (rc == SG_OK) {
+      *out = h;
+      return SG_OK;
+    }
+    const std::string msg = g_last_error;
+    sg_free(h);
+    if (rc != SG_ERR_OOM || !blocks) return fail(rc, msg);
   }
-  *out = h;
-  return SG_OK;
+  return fail(SG_ERR_OOM, "out of memory");
 }
 
 int sg_dims(const sg_handle* h, int sys, int* N, int* P, int* L) {
@@ -1041,14 +1122,22 @@ int sg_nnz(const sg_handle* h, int sys, long long* nnz_A, long long* nnz_G) {
 int sg_matvec(sg_handle* h, int sys, const double* X, double* Y, void* stream) {
   System* s = get_sys(h, sys);
   if (!s || !X || !Y) return fail(SG_ERR_ARG, "bad handle, system index or pointer");
-  return launch_matvec_f64(*s, X, Y, 1.0, nullptr, 0.0, (cudaStream_t)stream);
+  cudaStream_t st = (cudaStream_t)stream;
+  if (!s->block64.ready) return launch_matvec_f64(*s, X, Y, 1.0, nullptr, 0.0, st);
+  return matvec_pooled<double>(
+      h, *s, st, [&](double* f) { return launch_matvec_f64(*s, X, Y, 1.0, nullptr, 0.0, st, nullptr, f); },
+      [&]() { return launch_matvec_pairs_f64(*s, X, Y, st); });
 }
 
 int sg_matvec_lowp(sg_handle* h, int sys, const float* X, float* Y, void* stream) {
   System* s = get_sys(h, sys);
   if (!s || !X || !Y) return fail(SG_ERR_ARG, "bad handle, system index or pointer");
   if (s->prm.precision == SG_FP64) return fail(SG_ERR_ARG, "system has no low-precision stack");
-  return launch_matvec_f32(*s, X, Y, 1.0f, nullptr, 0.0f, (cudaStream_t)stream);
+  cudaStream_t st = (cudaStream_t)stream;
+  if (!s->block32.ready) return launch_matvec_f32(*s, X, Y, 1.0f, nullptr, 0.0f, st);
+  return matvec_pooled<float>(
+      h, *s, st, [&](float* f) { return launch_matvec_f32(*s, X, Y, 1.0f, nullptr, 0.0f, st, nullptr, f); },
+      [&]() { return launch_matvec_pairs_f32(*s, X, Y, st); });
 }
 
 int sg_precond_apply(sg_handle* h, int sys, const double* R, double* Z, void* stream) {
@@ -1126,7 +1215,15 @@ int sg_op_info(const sg_handle* h, int sys, long long* info, char* msg, int msg_
   System* s = get_sys(h, sys);
   if (!s || !info) return fail(SG_ERR_ARG, "bad handle, system index or pointer");
   const TileOp* ops[2] = {&s->tile64, &s->tile32};
+  const BlockOp* blk[2] = {&s->block64, &s->block32};
   for (int i = 0; i < 2; ++i) {
+    if (blk[i]->ready) {
+      info[4 * i + 0] = 3;
+      info[4 * i + 1] = blk[i]->TS;
+      info[4 * i + 2] = (long long)blk[i]->smem;
+      info[4 * i + 3] = blk[i]->nb;
+      continue;
+    }
     info[4 * i + 0] = ops[i]->ready ? 2 : 1;
     info[4 * i + 1] = ops[i]->ready ? ops[i]->kappa : 0;
     info[4 * i + 2] = ops[i]->ready ? (long long)ops[i]->smem : 0;
@@ -1238,6 +1335,7 @@ void sg_free(sg_handle* h) {
   if (!h) return;
   for (auto* s : h->sys) free_system(s);
   for (auto& e : h->timer.ev) cudaEventDestroy(e);
+  if (h->pool) cudaMemPoolDestroy(h->pool);
   delete h;
 }
 

@@ -267,6 +267,18 @@ struct TilePlan {
   std::vector<unsigned char> side;
 };
 
+// Block-stencil operator (k_apply_block.cu): per 32 nodes and edge block the tiles of its P x P
+// blocks in the round-robin order, the (round, range) table, and the products of one application
+// (5 x N x P) that the second kernel adds.
+struct BlockOp {
+  bool ready = false;
+  int elem = 0, TS = 0, nb = 0, rounds = 0, ntile = 0, nval = 0, row_tiles = 0, slots = 0, grid = 0;
+  size_t smem = 0, bytes = 0;
+  DBuf<int> table, tkind, err;
+  DBuf<double> k64, f64;
+  DBuf<float> k32, f32;
+};
+
 // ------------------------------------------------------------------ per-system state
 
 struct System {
@@ -295,6 +307,8 @@ struct System {
   DBuf<double> ent_g;
   DBuf<float> ent_g_f32;
   TileOp tile64, tile32;       // row-tiled operator in FP64 / FP32 (when built)
+  BlockOp block64, block32;    // block-stencil operator in FP64 / FP32 (when built)
+  bool lean = false;           // set up again without the block-stencil operator (out of memory)
   std::string tile_msg;        // why a row-tiled operator was not built (empty if it was)
   // device: preconditioner
   int nfac = 0;                // number of factor sets (1 for mean, P for field split)
@@ -395,6 +409,7 @@ struct System {
 struct sg_handle {
   std::vector<sg::System*> sys;
   int device = 0;
+  cudaMemPool_t pool = nullptr;  // scratch of sg_matvec calls (block-stencil operator), by stream
   sg::Timer timer;
 };
 
@@ -427,10 +442,17 @@ int launch_cast_f64(const float* src, double* dst, size_t n, cudaStream_t st);
 int launch_transpose(const double* src, double* dst, size_t rows, int cols, cudaStream_t st);
 
 // Y = alpha * K X + beta * B  (B may be null when beta == 0)
+// ``scratch``: block_scratch_elems values for the block-stencil form; null: the system's own, for
+// callers that use the system's workspace anyway (one at a time).
 int launch_matvec_f64(const System& s, const double* X, double* Y, double alpha, const double* B,
-                      double beta, cudaStream_t st, const int* done = nullptr);
+                      double beta, cudaStream_t st, const int* done = nullptr,
+                      double* scratch = nullptr);
 int launch_matvec_f32(const System& s, const float* X, float* Y, float alpha, const float* B,
-                      float beta, cudaStream_t st, const int* done = nullptr);
+                      float beta, cudaStream_t st, const int* done = nullptr,
+                      float* scratch = nullptr);
+// The operator by the pair kernel from the FP64 stack, which every system keeps.
+int launch_matvec_pairs_f64(const System& s, const double* X, double* Y, cudaStream_t st);
+int launch_matvec_pairs_f32(const System& s, const float* X, float* Y, cudaStream_t st);
 
 int precond_apply_f64(System& s, const double* R, double* Z, cudaStream_t st,
                       const int* done = nullptr);
@@ -473,6 +495,15 @@ void free_tile_op(TileOp& op);
 template <typename T>
 int launch_tile_op(const System& s, const TileOp& op, const T* X, T* Y, T alpha, const T* B,
                    T beta, cudaStream_t st, const int* done);
+
+// Block-stencil operator (k_apply_block.cu)
+size_t block_scratch_elems(const System& s);
+size_t block_op_bytes(const System& s, int elem);
+int build_block_op(System& s, BlockOp& op, int elem, cudaStream_t st);
+void free_block_op(BlockOp& op);
+template <typename T>
+int launch_block_op(const System& s, const BlockOp& op, const T* X, T* Y, T alpha, const T* B,
+                    T beta, T* scratch, cudaStream_t st, const int* done);
 
 // Krylov launchers (k_krylov.cu)
 int k_norm(System& s, size_t n, const double* r, double* out, cudaStream_t st);

@@ -262,7 +262,7 @@ def sg_op_info(h: SGHandle, sys: int = 0):
     info = (ctypes.c_longlong * 8)()
     msg = ctypes.create_string_buffer(512)
     _check(load_library().sg_op_info(h.raw, sys, info, msg, 512))
-    names = {0: "none", 1: "pairs", 2: "tile"}
+    names = {0: "none", 1: "pairs", 2: "tile", 3: "block"}
     out = {}
     for i, key in enumerate(("fp64", "fp32")):
         out[key] = {"kernel": names[int(info[4 * i])], "kappa": int(info[4 * i + 1]),
