@@ -22,31 +22,43 @@ constexpr int kBChunk = 128;       // batch rows staged per pass (kBChunk * kMax
 constexpr int kSplit = 152;        // CTAs of the split-K hidden-layer back-propagation
 constexpr int kJT = 32;            // output units per split-K step
 
-__global__ void small_fwd_kernel(int in, int h1, int h2, const float* __restrict__ Z,
-                                 const float* __restrict__ mu, const float* __restrict__ sd,
-                                 const float* __restrict__ P, int oW1, int ob1, int oW2, int ob2,
-                                 float* __restrict__ Zh, float* __restrict__ H1,
-                                 float* __restrict__ H2) {
-  __shared__ float zs[kMaxIn], a1[kMaxH1];
-  const int b = blockIdx.x, t = threadIdx.x;
-  if (t < in) {
-    float v = (Z[(size_t)b * in + t] - mu[t]) / sd[t];
-    zs[t] = v;
-    Zh[(size_t)b * in + t] = v;
+// Hidden layers of kFwdRows samples per CTA: W2 staged once in shared memory (rows padded by one
+// against bank conflicts), a thread per (sample, unit).
+constexpr int kFwdRows = 4;
+
+__global__ void __launch_bounds__(256) small_fwd_kernel(
+    int B, int in, int h1, int h2, const float* __restrict__ Z, const float* __restrict__ mu,
+    const float* __restrict__ sd, const float* __restrict__ P, int oW1, int ob1, int oW2, int ob2,
+    float* __restrict__ Zh, float* __restrict__ H1, float* __restrict__ H2) {
+  __shared__ float w2[kMaxH2 * (kMaxH1 + 1)], zs[kFwdRows][kMaxIn], a1[kFwdRows][kMaxH1];
+  const int b0 = blockIdx.x * kFwdRows, rows = min(kFwdRows, B - b0);
+  for (int t = threadIdx.x; t < h2 * h1; t += blockDim.x) {
+    const int q = t / h1, i = t - q * h1;
+    w2[q * (h1 + 1) + i] = P[oW2 + t];
+  }
+  for (int t = threadIdx.x; t < rows * in; t += blockDim.x) {
+    const int r = t / in, i = t - r * in;
+    const float v = (Z[(size_t)b0 * in + t] - mu[i]) / sd[i];
+    zs[r][i] = v;
+    Zh[(size_t)b0 * in + t] = v;
   }
   __syncthreads();
-  if (t < h1) {
-    float s = P[ob1 + t];
-    for (int i = 0; i < in; ++i) s = fmaf(P[oW1 + t * in + i], zs[i], s);
-    float v = tanhf(s);
-    a1[t] = v;
-    H1[(size_t)b * h1 + t] = v;
+  for (int t = threadIdx.x; t < rows * h1; t += blockDim.x) {
+    const int r = t / h1, u = t - r * h1;
+    float s = P[ob1 + u];
+    for (int i = 0; i < in; ++i) s = fmaf(P[oW1 + u * in + i], zs[r][i], s);
+    const float v = tanhf(s);
+    a1[r][u] = v;
+    H1[(size_t)b0 * h1 + t] = v;
   }
   __syncthreads();
-  if (t < h2) {
-    float s = P[ob2 + t];
-    for (int i = 0; i < h1; ++i) s = fmaf(P[oW2 + t * h1 + i], a1[i], s);
-    H2[(size_t)b * h2 + t] = tanhf(s);
+  for (int t = threadIdx.x; t < rows * h2; t += blockDim.x) {
+    const int r = t / h2, u = t - r * h2;
+    const float* w = w2 + u * (h1 + 1);
+    float s = P[ob2 + u];
+#pragma unroll 8
+    for (int i = 0; i < h1; ++i) s = fmaf(w[i], a1[r][i], s);
+    H2[(size_t)b0 * h2 + t] = tanhf(s);
   }
 }
 
@@ -178,7 +190,7 @@ __global__ void __launch_bounds__(256) dh2_partial_kernel(
         for (int q = 0; q < 4; ++q) acc[i][q] = fmaf(a[i], c[q], acc[i][q]);
     }
   }
-  float* o = part + (size_t)blockIdx.x * kMaxBatch * kMaxH2;
+  float* o = part + (size_t)blockIdx.x * B * kMaxH2;
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -188,60 +200,75 @@ __global__ void __launch_bounds__(256) dh2_partial_kernel(
     }
 }
 
-__global__ void dh2_final_kernel(int B, int h2, int nsplit, const float* __restrict__ part,
-                                 float* __restrict__ dH2) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= B * h2) return;
-  int b = t / h2, k = t - b * h2;
+// Per sample: dH2 = the sum of the split partials (four groups of splits, added in a fixed order),
+// dA2 = dH2 * (1 - h2^2), dH1 = W2^T dA2, dA1 = dH1 * (1 - h1^2).
+__global__ void __launch_bounds__(256) small_bwd_kernel(int B, int h1, int h2, int nsplit,
+                                                        const float* __restrict__ part,
+                                                        const float* __restrict__ P, int oW2,
+                                                        const float* __restrict__ H1,
+                                                        const float* __restrict__ H2,
+                                                        float* __restrict__ dA2,
+                                                        float* __restrict__ dA1) {
+  __shared__ float ps[4][kMaxH2], a2[kMaxH2];
+  const int b = blockIdx.x, t = threadIdx.x, k = t & 63, g = t >> 6;
   float s = 0.f;
-  for (int c = 0; c < nsplit; ++c) s += part[(size_t)c * kMaxBatch * kMaxH2 + (size_t)b * kMaxH2 + k];
-  dH2[t] = s;
-}
-
-// Per sample: dA2 = dH2 * (1 - h2^2), dH1 = W2^T dA2, dA1 = dH1 * (1 - h1^2).
-__global__ void small_bwd_kernel(int h1, int h2, const float* __restrict__ P, int oW2,
-                                 const float* __restrict__ dH2, const float* __restrict__ H1,
-                                 const float* __restrict__ H2, float* __restrict__ dA2,
-                                 float* __restrict__ dA1) {
-  __shared__ float a2[kMaxH2];
-  const int b = blockIdx.x, t = threadIdx.x;
+  const float* p = part + (size_t)b * kMaxH2 + k;
+#pragma unroll 8
+  for (int c = g; c < nsplit; c += 4) s += p[(size_t)c * B * kMaxH2];
+  ps[g][k] = s;
+  __syncthreads();
   if (t < h2) {
-    float hv = H2[(size_t)b * h2 + t];
-    float v = dH2[(size_t)b * h2 + t] * (1.f - hv * hv);
+    const float hv = H2[(size_t)b * h2 + t];
+    const float v = ((ps[0][t] + ps[1][t]) + (ps[2][t] + ps[3][t])) * (1.f - hv * hv);
     a2[t] = v;
     dA2[(size_t)b * h2 + t] = v;
   }
   __syncthreads();
   if (t < h1) {
-    float s = 0.f;
-    for (int q = 0; q < h2; ++q) s = fmaf(P[oW2 + q * h1 + t], a2[q], s);
-    float hv = H1[(size_t)b * h1 + t];
-    dA1[(size_t)b * h1 + t] = s * (1.f - hv * hv);
+    float d = 0.f;
+#pragma unroll 8
+    for (int q = 0; q < h2; ++q) d = fmaf(P[oW2 + q * h1 + t], a2[q], d);
+    const float hv = H1[(size_t)b * h1 + t];
+    dA1[(size_t)b * h1 + t] = d * (1.f - hv * hv);
   }
 }
 
 // Gradients of the small layers: gW2 = dA2^T H1, gb2, gW1 = dA1^T Zh, gb1 (sums over the batch).
-__global__ void small_wgrad_kernel(int B, int in, int h1, int h2, const float* __restrict__ Zh,
-                                   const float* __restrict__ H1, const float* __restrict__ dA1,
-                                   const float* __restrict__ dA2, float* __restrict__ G, int oW1,
-                                   int ob1, int oW2, int ob2) {
-  const int nW2 = h2 * h1, nW1 = h1 * in;
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  float s = 0.f;
-  if (t < nW2) {
-    int q = t / h1, i = t - q * h1;
-    for (int b = 0; b < B; ++b) s = fmaf(dA2[(size_t)b * h2 + q], H1[(size_t)b * h1 + i], s);
-    G[oW2 + t] = s;
-  } else if ((t -= nW2) < h2) {
-    for (int b = 0; b < B; ++b) s += dA2[(size_t)b * h2 + t];
-    G[ob2 + t] = s;
-  } else if ((t -= h2) < nW1) {
-    int q = t / in, i = t - q * in;
-    for (int b = 0; b < B; ++b) s = fmaf(dA1[(size_t)b * h1 + q], Zh[(size_t)b * in + i], s);
-    G[oW1 + t] = s;
-  } else if ((t -= nW1) < h1) {
-    for (int b = 0; b < B; ++b) s += dA1[(size_t)b * h1 + t];
-    G[ob1 + t] = s;
+// CTA r: row r of W2 and b2[r] (r < h2), or row r - h2 of W1 and b1: out[i] = sum_b d[b] in[b, i],
+// the batch over the groups of threads that hold one column each, the groups' sums added in a
+// fixed order.  (One thread per weight with the whole batch in sequence took 42 us at B = 256.)
+__global__ void __launch_bounds__(512) small_wgrad_kernel(
+    int B, int in, int h1, int h2, const float* __restrict__ Zh, const float* __restrict__ H1,
+    const float* __restrict__ dA1, const float* __restrict__ dA2, float* __restrict__ G, int oW1,
+    int ob1, int oW2, int ob2) {
+  __shared__ float ps[512], pb[512];
+  const bool two = (int)blockIdx.x < h2;
+  const int r = two ? blockIdx.x : blockIdx.x - h2;
+  const int w = two ? h1 : in, ld = two ? h2 : h1;
+  const float* d = (two ? dA2 : dA1) + r;
+  const float* x = two ? H1 : Zh;
+  const int groups = 512 / w, g = threadIdx.x / w, i = threadIdx.x - g * w;
+  float s = 0.f, sb = 0.f;
+  if (g < groups) {
+#pragma unroll 8
+    for (int b = g; b < B; b += groups) {
+      const float dv = d[(size_t)b * ld];
+      s = fmaf(dv, x[(size_t)b * w + i], s);
+      sb += dv;
+    }
+  }
+  ps[threadIdx.x] = s;
+  pb[threadIdx.x] = sb;
+  __syncthreads();
+  if ((int)threadIdx.x < w) {
+    float v = 0.f;
+    for (int q = 0; q < groups; ++q) v += ps[q * w + threadIdx.x];
+    G[(two ? oW2 : oW1) + r * w + threadIdx.x] = v;
+  }
+  if (threadIdx.x == 0) {
+    float v = 0.f;
+    for (int q = 0; q < groups; ++q) v += pb[q * w];
+    G[(two ? ob2 : ob1) + r] = v;
   }
 }
 
@@ -378,12 +405,9 @@ struct sgnet {
   int oW1 = 0, ob1 = 0, oW2 = 0, ob2 = 0, oW3 = 0, ob3 = 0;
   long long np = 0, step = 0;
   int frozen_out = 0;        // 1: Adam leaves the output layer (W3, b3) as set_basis left it
-  sg::DBuf<float> P, G, M, V, mu, sd, Zh, H1, H2, dY, dH2, dA2, dA1, part, lpart, loss, Ytmp;
+  sg::DBuf<float> P, G, M, V, mu, sd, Zh, H1, H2, dY, dA2, dA1, part, lpart, loss;
   sg::DBuf<__nv_bfloat16> W3h;
-  // tensor-core back-propagation: W3 transposed (64 x outp) and dY (max batch x outp) in BF16,
-  // outp = out rounded up to a multiple of 64
-  int outp = 0;
-  sg::DBuf<__nv_bfloat16> W3hT, dYh;
+  sg::DBuf<__nv_bfloat16> W3c;  // W3 in BF16 tiles for the tensor-core training pass
   sg::DBuf<int> err;         // raised by a tensor-core kernel whose MMA completion timed out
 };
 
@@ -391,11 +415,10 @@ using namespace sg;
 
 static int net_release(sgnet* n) {
   DBuf<float>* bs[] = {&n->P, &n->G, &n->M, &n->V, &n->mu, &n->sd, &n->Zh, &n->H1, &n->H2,
-                       &n->dY, &n->dH2, &n->dA2, &n->dA1, &n->part, &n->lpart, &n->loss, &n->Ytmp};
+                       &n->dY, &n->dA2, &n->dA1, &n->part, &n->lpart, &n->loss};
   for (auto* b : bs) b->release();
   n->W3h.release();
-  n->W3hT.release();
-  n->dYh.release();
+  n->W3c.release();
   n->err.release();
   return SG_OK;
 }
@@ -415,14 +438,15 @@ static int refresh_bf16(sgnet* n, cudaStream_t st) {
   if (!n->bf16) return SG_OK;
   to_bf16_kernel<<<608, 256, 0, st>>>((size_t)n->out * n->h2, n->P.p + n->oW3, n->W3h.p);
   SG_TRY(check_launch("to_bf16"));
-  if (n->W3hT.p) SG_TRY(launch_w3t_bf16(n->out, n->outp, n->h2, n->P.p + n->oW3, n->W3hT.p, st));
+  if (n->W3c.p) SG_TRY(launch_w3_tiles(n->out, n->h2, n->P.p + n->oW3, n->W3c.p, st));
   return SG_OK;
 }
 
 static const __nv_bfloat16* w3h(const sgnet* n) { return n->bf16 ? n->W3h.p : nullptr; }
 
 static int forward_hidden(sgnet* n, const float* Z, int B, cudaStream_t st) {
-  small_fwd_kernel<<<B, 128, 0, st>>>(n->in, n->h1, n->h2, Z, n->mu.p, n->sd.p, n->P.p, n->oW1,
+  small_fwd_kernel<<<(B + kFwdRows - 1) / kFwdRows, 256, 0, st>>>(
+      B, n->in, n->h1, n->h2, Z, n->mu.p, n->sd.p, n->P.p, n->oW1,
                                       n->ob1, n->oW2, n->ob2, n->Zh.p, n->H1.p, n->H2.p);
   return check_launch("small_fwd");
 }
@@ -481,18 +505,15 @@ int sgnet_create(int in_dim, int h1, int h2, int out_dim, int max_batch, int bf1
   A(n->P, n->np); A(n->G, n->np); A(n->M, n->np); A(n->V, n->np);
   A(n->mu, in_dim); A(n->sd, in_dim);
   A(n->Zh, B * in_dim); A(n->H1, B * h1); A(n->H2, B * h2); A(n->dY, B * out_dim);
-  A(n->dH2, B * h2); A(n->dA2, B * h2); A(n->dA1, B * h1);
-  A(n->part, (size_t)kSplit * kMaxBatch * kMaxH2);
-  // loss partials: one per CTA of the SIMT output kernel, or per 128 x 128 tile of the
-  // tensor-core one
-  A(n->lpart, (size_t)(out_dim + kOutThreads - 1) / kOutThreads * ((B + 127) / 128));
+  A(n->dA2, B * h2); A(n->dA1, B * h1);
+  // split partials of dH2: kSplit per sample, or in a tensor-core training pass kTcTrainCtas per
+  // (up to) 128 samples
+  A(n->part, std::max((size_t)kSplit * B, (size_t)kTcTrainCtas * std::min<size_t>(B, 128)) * kMaxH2);
+  // loss partials: one per CTA of the SIMT output kernel or of the tensor-core training pass
+  A(n->lpart, std::max((size_t)(out_dim + kOutThreads - 1) / kOutThreads, (size_t)kTcTrainCtas));
   A(n->loss, 1);
   if (rc == SG_OK && n->bf16) rc = n->W3h.alloc((size_t)out_dim * h2);
-  if (rc == SG_OK && n->bf16 && h2 <= kMaxH2) {
-    n->outp = (out_dim + 63) / 64 * 64;
-    rc = n->W3hT.alloc((size_t)64 * n->outp);
-    if (rc == SG_OK) rc = n->dYh.alloc(B * n->outp);
-  }
+  if (rc == SG_OK && n->bf16 && h2 <= kMaxH2) rc = n->W3c.alloc(w3_tiles_elems(out_dim));
   if (rc == SG_OK) rc = n->err.alloc(1);
   if (rc == SG_OK && cudaMemset(n->err.p, 0, sizeof(int)) != cudaSuccess)
     rc = fail(SG_ERR_CUDA, "cudaMemset of the error word failed");
@@ -577,8 +598,8 @@ int sgnet_forward(sgnet* n, const float* Z, int B, float* Y, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   SG_TRY(forward_hidden(n, Z, B, st));
   if (use_tc(n))
-    return launch_out_tc(0, B, n->h2, n->out, n->H2.p, n->W3h.p, n->P.p + n->ob3, Y, nullptr,
-                         nullptr, nullptr, 0, nullptr, n->err.p, st, nullptr);
+    return launch_out_tc(B, n->h2, n->out, n->H2.p, n->W3h.p, n->P.p + n->ob3, Y, nullptr,
+                         n->err.p, st);
   out_kernel<0, float><<<(n->out + kOutThreads - 1) / kOutThreads, kOutThreads, 0, st>>>(
       B, n->h2, n->out, n->H2.p, n->P.p + n->oW3, w3h(n), n->P.p + n->ob3, Y, nullptr, nullptr,
       nullptr, nullptr, nullptr);
@@ -591,8 +612,8 @@ int sgnet_predict(sgnet* n, const float* Z, int B, double* X, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   SG_TRY(forward_hidden(n, Z, B, st));
   if (use_tc(n))
-    return launch_out_tc(0, B, n->h2, n->out, n->H2.p, n->W3h.p, n->P.p + n->ob3, nullptr, X,
-                         nullptr, nullptr, 0, nullptr, n->err.p, st, nullptr);
+    return launch_out_tc(B, n->h2, n->out, n->H2.p, n->W3h.p, n->P.p + n->ob3, nullptr, X,
+                         n->err.p, st);
   out_kernel<0, double><<<(n->out + kOutThreads - 1) / kOutThreads, kOutThreads, 0, st>>>(
       B, n->h2, n->out, n->H2.p, n->P.p + n->oW3, w3h(n), n->P.p + n->ob3, X, nullptr, nullptr,
       nullptr, nullptr, nullptr);
@@ -606,38 +627,32 @@ int sgnet_loss_grad(sgnet* n, const float* Z, const float* T, int B, float* loss
   SG_TRY(forward_hidden(n, Z, B, st));
   int nblk = (n->out + kOutThreads - 1) / kOutThreads;
   const bool tc = use_tc(n) && n->frozen_out;
+  int nsplit = kSplit;
   if (tc) {
-    // the output layer is fixed: only the residual gradient dY (BF16) and the loss are needed
-    SG_TRY(launch_out_tc(1, B, n->h2, n->out, n->H2.p, n->W3h.p, n->P.p + n->ob3, nullptr,
-                         nullptr, T, n->dYh.p, n->outp, n->lpart.p, n->err.p, st, &nblk));
+    // the output layer is fixed: residual, loss and back-propagation in one pass over T
+    SG_TRY(launch_train_tc(B, n->h2, n->out, n->H2.p, n->W3c.p, n->P.p + n->ob3, T, n->part.p,
+                           n->lpart.p, n->err.p, st, &nsplit, &nblk));
   } else {
     out_kernel<1, float><<<nblk, kOutThreads, 0, st>>>(B, n->h2, n->out, n->H2.p,
                                                         n->P.p + n->oW3, w3h(n), n->P.p + n->ob3,
                                                         nullptr, T, n->dY.p, n->G.p + n->oW3,
                                                         n->G.p + n->ob3, n->lpart.p);
     SG_TRY(check_launch("out_grad"));
-  }
-  loss_final_kernel<<<1, 256, 0, st>>>(nblk, n->lpart.p, (float)B * (float)n->out, n->loss.p);
-  SG_TRY(check_launch("loss_final"));
-  int nsplit = kSplit;
-  if (tc) {
-    SG_TRY(launch_dh2_tc(B, n->outp, n->dYh.p, n->W3hT.p, n->part.p, (size_t)kMaxBatch * kMaxH2,
-                         kMaxH2, kSplit, n->err.p, st, &nsplit));
-  } else {
     dim3 g(kSplit, (B + 63) / 64);
     dh2_partial_kernel<<<g, 256, 0, st>>>(B, n->h2, n->out, n->dY.p, n->P.p + n->oW3, w3h(n),
                                           n->part.p);
     SG_TRY(check_launch("dh2_partial"));
   }
-  dh2_final_kernel<<<(B * n->h2 + 255) / 256, 256, 0, st>>>(B, n->h2, nsplit, n->part.p, n->dH2.p);
-  SG_TRY(check_launch("dh2_final"));
-  small_bwd_kernel<<<B, 128, 0, st>>>(n->h1, n->h2, n->P.p, n->oW2, n->dH2.p, n->H1.p, n->H2.p,
-                                      n->dA2.p, n->dA1.p);
+  if (loss) {  // only a caller that asks for the loss has it summed
+    loss_final_kernel<<<1, 256, 0, st>>>(nblk, n->lpart.p, (float)B * (float)n->out, n->loss.p);
+    SG_TRY(check_launch("loss_final"));
+  }
+  small_bwd_kernel<<<B, 256, 0, st>>>(B, n->h1, n->h2, nsplit, n->part.p, n->P.p, n->oW2, n->H1.p,
+                                      n->H2.p, n->dA2.p, n->dA1.p);
   SG_TRY(check_launch("small_bwd"));
-  int nsmall = n->h2 * n->h1 + n->h2 + n->h1 * n->in + n->h1;
-  small_wgrad_kernel<<<(nsmall + 127) / 128, 128, 0, st>>>(B, n->in, n->h1, n->h2, n->Zh.p, n->H1.p,
-                                                           n->dA1.p, n->dA2.p, n->G.p, n->oW1,
-                                                           n->ob1, n->oW2, n->ob2);
+  small_wgrad_kernel<<<n->h2 + n->h1, 512, 0, st>>>(B, n->in, n->h1, n->h2, n->Zh.p, n->H1.p,
+                                                    n->dA1.p, n->dA2.p, n->G.p, n->oW1, n->ob1,
+                                                    n->oW2, n->ob2);
   SG_TRY(check_launch("small_wgrad"));
   if (loss) {
     SG_CUDA(cudaMemcpyAsync(loss, n->loss.p, sizeof(float), cudaMemcpyDeviceToHost, st));
@@ -653,9 +668,10 @@ int sgnet_adam_step(sgnet* n, float lr, void* stream) {
   float c1 = (float)(1.0 - std::pow(0.9, (double)n->step));
   float c2 = (float)(1.0 - std::pow(0.999, (double)n->step));
   const size_t nupd = n->frozen_out ? (size_t)n->oW3 : (size_t)n->np;  // W3, b3 come last
-  adam_kernel<<<608, 256, 0, st>>>(nupd, n->P.p, n->G.p, n->M.p, n->V.p, lr, c1, c2);
+  const int grid = (int)std::min<size_t>(608, (nupd + 255) / 256);
+  adam_kernel<<<grid, 256, 0, st>>>(nupd, n->P.p, n->G.p, n->M.p, n->V.p, lr, c1, c2);
   SG_TRY(check_launch("adam"));
-  return refresh_bf16(n, st);
+  return n->frozen_out ? SG_OK : refresh_bf16(n, st);  // a fixed W3 keeps its copies
 }
 
 int sgnet_train_step(sgnet* n, const float* Z, const float* T, int B, float lr, float* loss,
