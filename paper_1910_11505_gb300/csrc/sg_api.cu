@@ -799,14 +799,13 @@ static int iteration(System& s, int j, int last_col) {
     double* zj = s.Z.p + (size_t)j * n;
     SG_TRY(precond_apply_f64(s, vj, zj, st, done));
     SG_TRY(launch_matvec_f64(s, zj, w, 1.0, nullptr, 0.0, st, done));
-  } else {
-    float* z32 = s.Z32.p + (size_t)j * n;
-    SG_TRY(k_to_f32(n, vj, s.mv32a.p, done, st));
-    SG_TRY(precond_apply_f32(s, s.mv32a.p, z32, st, done));
-    SG_TRY(launch_matvec_f32(s, z32, s.mv32b.p, 1.0f, nullptr, 0.0f, st, done));
-    SG_TRY(k_to_f64(n, s.mv32b.p, w, done, st));
+    return k_arnoldi(s, n, j, last_col, nullptr, st);
   }
-  return k_arnoldi(s, n, j, last_col, st);
+  // mixed: v_j's FP32 copy is in mv32a (left by the cycle's start or the step before)
+  float* z32 = s.Z32.p + (size_t)j * n;
+  SG_TRY(precond_apply_f32(s, s.mv32a.p, z32, st, done));
+  SG_TRY(launch_matvec_f32(s, z32, s.mv32b.p, 1.0f, nullptr, 0.0f, st, done));
+  return k_arnoldi(s, n, j, last_col, s.mv32b.p, st);
 }
 
 // r = F - K x, beta = ||r||, mirrored to host with the cycle flags.  For the initial iterate

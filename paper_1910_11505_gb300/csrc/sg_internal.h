@@ -509,10 +509,8 @@ int k_norm(System& s, size_t n, const double* r, double* out, cudaStream_t st);
 // *flag != 0 afterwards iff x[0..n) is all zero (the flag then skips kernels given it as done).
 int k_zero_flag(System& s, size_t n, const double* x, int* flag, cudaStream_t st);
 int k_init_cycle(System& s, size_t n, const double* r, cudaStream_t st);
-int k_arnoldi(System& s, size_t n, int j, int last_col, cudaStream_t st);
+int k_arnoldi(System& s, size_t n, int j, int last_col, const float* w32, cudaStream_t st);
 int k_finish_cycle(System& s, size_t n, double* x, bool z32, cudaStream_t st);
-int k_to_f32(size_t n, const double* src, float* dst, const int* flags, cudaStream_t st);
-int k_to_f64(size_t n, const float* src, double* dst, const int* flags, cudaStream_t st);
 int krylov_red_blocks();
 int krylov_max_basis();
 
