@@ -85,7 +85,6 @@ __global__ void __launch_bounds__((kBlockMaxWarps + 1) * 32) block_edge_kernel(
     BlockArgs g, const int* __restrict__ table, const int* __restrict__ tkind,
     const T* __restrict__ K, const T* __restrict__ X, T* __restrict__ F,
     const int* __restrict__ done, int* __restrict__ err) {
-  if (done != nullptr && *done) return;
   constexpr int kPair = TS * TS, kDiag = TS * (TS + 1) / 2;
   constexpr unsigned kSlot = kPair * kBR * sizeof(T);
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -122,13 +121,20 @@ __global__ void __launch_bounds__((kBlockMaxWarps + 1) * 32) block_edge_kernel(
   // two before; once the tile is issued (every earlier use of the slot is over) it does.
   volatile unsigned* vissued = reinterpret_cast<volatile unsigned*>(s_fail + 1);
 
-  if (w == nb) {  // producer
+  if (w == nb) {  // producer: the first ring of tiles before the kernel before this one has ended
     if (lane == 0) {
       unsigned cnt = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
         const T* src = K + (size_t)it * g.item_elems;
         for (int s = 0; s < g.ntile; ++s, ++cnt) {
+          if (cnt == (unsigned)g.slots) {
+            pdl_wait();
+            if (done != nullptr && *done) {
+              ok = false;
+              break;
+            }
+          }
           const int slot = (int)(cnt & slot_mask);
           if (cnt >= (unsigned)g.slots &&
               !mbar_wait_bounded(&empty[slot], ((cnt >> slot_log) - 1u) & 1u)) {
@@ -156,6 +162,8 @@ __global__ void __launch_bounds__((kBlockMaxWarps + 1) * 32) block_edge_kernel(
     return;
   }
 
+  pdl_wait();
+  if (done != nullptr && *done) return;
   // consumers: thread tid stages elements tid, tid + nthr, ... of an item's 32 x P differences
   auto bar = [&]() { asm volatile("bar.sync 1, %0;\n" ::"r"(nthr) : "memory"); };
   T xi[TS], xj[TS];
@@ -254,6 +262,8 @@ __global__ void __launch_bounds__((kBlockMaxWarps + 1) * 32) block_edge_kernel(
         o[q] = D[b * kBLd + r];
       }
     }
+    // (the next kernel's CTAs do not share the SMs with more than the last items)
+    if (it + (int)gridDim.x >= nitems) pdl_trigger();
   }
 }
 
@@ -269,6 +279,8 @@ __global__ void __launch_bounds__(256) block_sum_kernel(int N, int m, int P,
                                                         const T* __restrict__ X, T* __restrict__ Y,
                                                         T alpha, const T* __restrict__ B, T beta,
                                                         const int* __restrict__ done) {
+  pdl_trigger();
+  pdl_wait();
   if (done != nullptr && *done) return;
   using W = BlockVec<T, V>;
   const unsigned NP = (unsigned)N * (unsigned)P;
@@ -560,20 +572,16 @@ int launch_block_op(const System& s, const BlockOp& op, const T* X, T* Y, T alph
                     (long long)op.nval * kBR, op.bytes > ((size_t)64 << 20) ? 1 : 0};
   auto kern = block_kernel<T>(op.TS);
   TimeScope ts(s.timer, sizeof(T) == 8 ? K_APPLY_F64 : K_APPLY_LOWP, st);
-  kern<<<op.grid, (op.nb + 1) * 32, op.smem, st>>>(g, op.table.p, op.tkind.p, block_store<T>(op), X,
-                                                  F, done, op.err.p);
-  SG_TRY(check_launch("block_edge"));
+  SG_TRY(launch_pdl(kern, dim3(op.grid), dim3((op.nb + 1) * 32), op.smem, st, g, (const int*)op.table.p,
+                    (const int*)op.tkind.p, (const T*)block_store<T>(op), X, F, done, op.err.p));
   // 16-byte accesses where every row starts on one
   constexpr int kV = 16 / sizeof(T);
   const auto addr = [](const void* p) { return reinterpret_cast<unsigned long long>(p); };
   const bool vec = s.P % kV == 0 && ((addr(X) | addr(Y) | addr(B) | addr(F)) & 15) == 0;
   const size_t n = (size_t)s.N * s.P / (vec ? kV : 1);
   const int grid = (int)std::min<size_t>((n + 255) / 256, 152 * 16);
-  if (vec)
-    block_sum_kernel<T, kV><<<grid, 256, 0, st>>>(s.N, s.pat.m, s.P, F, X, Y, alpha, B, beta, done);
-  else
-    block_sum_kernel<T, 1><<<grid, 256, 0, st>>>(s.N, s.pat.m, s.P, F, X, Y, alpha, B, beta, done);
-  return check_launch("block_sum");
+  return launch_pdl(vec ? block_sum_kernel<T, kV> : block_sum_kernel<T, 1>, dim3(grid), dim3(256), 0, st,
+                    s.N, s.pat.m, s.P, (const T*)F, X, Y, alpha, B, beta, done);
 }
 
 template int launch_block_op<double>(const System&, const BlockOp&, const double*, double*, double,

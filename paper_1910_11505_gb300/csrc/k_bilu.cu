@@ -303,138 +303,206 @@ __global__ void __launch_bounds__(256) fg_factor_kernel(int m, int Q, int c,
   }
 }
 
-// Lanes per node in the solve kernels (the rows of a block, in whole warps) and threads per CTA:
-// one node of 3 or 4 warps, else 128 threads holding 2 or 4 nodes.
-__host__ __device__ constexpr int fg_lanes(int Q) {
-  return Q > 96 ? 128 : Q > 64 ? 96 : Q > 32 ? 64 : 32;
-}
-__host__ __device__ constexpr int fg_cta_threads(int Q) { return fg_lanes(Q) == 96 ? 96 : 128; }
-
 // Block storage of the solve kernels.  FP32 / FP64 factors: each Q x Q block column-major.
 // BF16 factors: columns in fours, (r, c) at ((c / 4) * Q + r) * 4 + (c & 3), the column count
-// rounded up to a multiple of four (Qc) with zero columns, so a lane reads four values of its
-// row in one 8-byte load and a warp's load covers 256 contiguous bytes.
+// rounded up to a multiple of four (Qc) with zero columns, so that a load of 8 bytes gives four
+// values of a row.
 template <typename TV>
 __host__ __device__ constexpr bool fg_quads() { return sizeof(TV) == 2; }
 __host__ __device__ inline int fg_qc(int Q) { return (Q + 3) & ~3; }
 
-// Row r of block blk times the vector v (Qc values, zero-padded): four partial sums.
-template <typename T, typename TV>
-__device__ __forceinline__ T fg_block_row_dot(const TV* __restrict__ blk, int Q, int r,
-                                              const T* v) {
-  T s0 = T(0), s1 = T(0), s2 = T(0), s3 = T(0);
-  if constexpr (fg_quads<TV>()) {
-    const uint2* b4 = reinterpret_cast<const uint2*>(blk) + r;
-    const int nq = fg_qc(Q) >> 2;
-#pragma unroll 21  // all of a row's loads in flight at once for up to 84 fields
-    for (int cq = 0; cq < nq; ++cq) {
-      const uint2 w = b4[(size_t)cq * Q];
-      const float2 u0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w.x));
-      const float2 u1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w.y));
-      s0 += (T)u0.x * v[4 * cq];
-      s1 += (T)u0.y * v[4 * cq + 1];
-      s2 += (T)u1.x * v[4 * cq + 2];
-      s3 += (T)u1.y * v[4 * cq + 3];
-    }
-  } else {
-    const TV* b = blk + r;
-    int cc = 0;
-#pragma unroll 2
-    for (; cc + 4 <= Q; cc += 4) {
-      s0 += (T)b[(size_t)cc * Q] * v[cc];
-      s1 += (T)b[(size_t)(cc + 1) * Q] * v[cc + 1];
-      s2 += (T)b[(size_t)(cc + 2) * Q] * v[cc + 2];
-      s3 += (T)b[(size_t)(cc + 3) * Q] * v[cc + 3];
-    }
-    for (; cc < Q; ++cc) s0 += (T)b[(size_t)cc * Q] * v[cc];
-  }
-  return (s0 + s1) + (s2 + s3);
-}
+// A block is Q rows x nc units (a unit: one value, or four of a row in BF16), unit-column by
+// unit-column.  ``groups`` x Q threads share a node: thread t takes row t % Q of the unit columns
+// t / Q + i * groups, so that they read a block as one contiguous stream whatever Q is; a CTA takes
+// as many nodes as fit in kFgThreads.
+constexpr int kFgThreads = 256;
+template <typename TV>
+__host__ __device__ inline int fg_units(int Q) { return fg_quads<TV>() ? fg_qc(Q) / 4 : Q; }
 
 // Whether neighbour slot sl (0..8, 4 = the node itself) takes part in a phase of colour c: the
 // forward sweep uses the slots of lower colours, the backward sweep the diagonal and the slots
 // of higher colours.  A neighbour's colour follows from the node's parities, so the set is the
 // same for every node of the launch.
-__device__ __forceinline__ bool fg_slot_used(int c, int sl, bool upper) {
+__host__ __device__ constexpr bool fg_slot_used(int c, int sl, bool upper) {
   if (sl == 4) return upper;
-  const int nc = fg_colour((c & 1) + sl % 3 - 1 + 2, (c >> 1) + sl / 3 - 1 + 2);
-  return upper ? nc > c : nc < c;
+  const int x = ((c & 1) + sl % 3 + 1) & 1, y = ((c >> 1) + sl / 3 + 1) & 1;
+  return upper ? x + 2 * y > c : x + 2 * y < c;
+}
+template <int C, bool UPPER>
+__host__ __device__ constexpr int fg_used() {
+  int n = 0;
+  for (int sl = 0; sl < 9; ++sl) n += fg_slot_used(C, sl, UPPER);
+  return n;
+}
+// Slot of the k-th used one.
+template <int C, bool UPPER>
+__host__ __device__ constexpr int fg_slot(int k) {
+  for (int sl = 0; sl < 9; ++sl)
+    if (fg_slot_used(C, sl, UPPER) && k-- == 0) return sl;
+  return 4;
 }
 
-// One colour of a sweep of a split (fields [f0, f0 + Q) of the N x P arrays).
+template <typename T>
+struct FgUnit { using type = T; };
+template <>
+struct FgUnit<__nv_bfloat16> { using type = uint2; };
+
+// One colour of a sweep of a split (fields [f0, f0 + Q) of the N x P arrays), npc nodes per CTA.
 //   forward (UPPER = false): y_i = r_i - sub_i - sum over the lower-colour slots of
 //     (L D^-1)_{i,slot} y_nb;
 //   backward (UPPER = true, in place): z_i = D_i^-1 y_i - sum over the higher-colour slots of
 //     (D^-1 U)_{i,slot} z_nb.
-// Each node is a group of lanes (lane r: row r of every block).  The Q values of every slot the
-// phase uses (the node's own y_i included in the backward sweep) are staged in shared memory
-// first, behind one barrier; then each lane streams its rows of those blocks.  Neighbours
-// outside the mesh have zero blocks and are staged as zero vectors.  No other node of the
-// colour reads node i, so writing it in place is safe.
-template <typename T, typename TV, bool UPPER>
-__global__ void __launch_bounds__(128) fg_phase_kernel(int m, int P, int Q, int f0, int c,
-                                                       const int* __restrict__ cstart_g,
-                                                       const TV* __restrict__ fac,
-                                                       const T* __restrict__ R,
-                                                       const T* __restrict__ sub, T* Y,
-                                                       const int* __restrict__ done) {
-  if (done != nullptr && *done) return;
+// The Q values of every slot the phase uses (the node's own y_i included in the backward sweep) are
+// staged in shared memory, negated except the own ones; neighbours outside the mesh have zero
+// blocks and are staged as zero vectors.  No other node of the colour reads node i, so writing it
+// in place is safe.  The threads that share a row add their sums at the end in a fixed order.
+//
+// Bound: HBM on large meshes (the factors are read once; in FP64 the FP64 pipe), latency on small
+// ones.  So a thread keeps B loads in flight, refilled one by one across the slots; where a colour
+// has too few nodes to fill the GPU with Q threads each, several groups of threads split the
+// columns too (a lane per row that walked all columns took 40 trips to memory per node at Q = 35);
+// and the first loads, which depend on no earlier kernel, are issued before the wait for the phase
+// before (programmatic launch).  Measured on one GB300, one application, against the kernel with
+// a lane per row: BF16 Q = 84, n = 256 1.39 ms (6.1 TB/s) against 1.46, n = 32 62 us against 130,
+// n = 4 40 against 63; FP32 Q = 35, n = 128 204 us against 573, n = 8 33 against 123; FP64 Q = 35,
+// n = 128 593 us against 784.
+template <typename T, typename TV, bool UPPER, int C, int B>
+__global__ void __launch_bounds__(kFgThreads, sizeof(T) == 4 && B > 8 ? 4 : 1)
+    fg_phase_kernel(int m, int P, int Q, int f0,
+                                                              int groups, int npc, int cnt,
+                                                              const int* __restrict__ cstart_g,
+                                                              const TV* __restrict__ fac,
+                                                              const T* __restrict__ R,
+                                                              const T* __restrict__ sub, T* Y,
+                                                              const int* __restrict__ done) {
+  constexpr int kUsed = fg_used<C, UPPER>();
+  using U = typename FgUnit<TV>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int G = fg_lanes(Q), npc = fg_cta_threads(Q) / G;
-  const int g = threadIdx.x / G, r = threadIdx.x % G;
-  const int c0 = cstart_g[c], cnt = cstart_g[c + 1] - c0;
-  const int idx = blockIdx.x * npc + g;
-  const bool live = idx < cnt;
-  const int pos = c0 + (live ? idx : cnt - 1);
-  int x, y;
-  {
-    const int cx = c & 1, cy = c >> 1, nx = (m - cx + 1) >> 1, q = pos - c0;
-    y = cy + 2 * (q / nx);
-    x = cx + 2 * (q % nx);
-  }
-  const int i = x + m * y;
-  const int Qc = fg_qc(Q);
-  const size_t QQ = (size_t)Q * (fg_quads<TV>() ? Qc : Q);
-  const TV* blocks = fac + (size_t)pos * 9 * QQ;
-  T* v = reinterpret_cast<T*>(smem_raw) + (size_t)g * 9 * Qc;  // one vector per used slot
-  int k = 0;
+  pdl_trigger();
+  const int nc = fg_units<TV>(Q), Qc = fg_qc(Q);
+  const int stride = groups * Q;  // threads of a node, and units between a thread's columns
+  const int nd = threadIdx.x / stride, t = threadIdx.x - nd * stride, g = t / Q, r = t - g * Q;
+  const int q = blockIdx.x * npc + nd;  // node of the colour
+  const bool live = nd < npc && q < cnt;
+  // unit columns of a block: this thread's, and the batches that the CTA walks them in
+  const int mine = live ? (nc - g + groups - 1) / groups : 0;
+  const int nch = ((nc + groups - 1) / groups + B - 1) / B;
+  constexpr int cx = C & 1, cy = C >> 1;
+  const int nx = (m - cx + 1) >> 1, qn = live ? q : 0;
+  const int y = cy + 2 * (qn / nx), x = cx + 2 * (qn % nx);
+  const int i = x + m * y, pos = cstart_g[C] + qn;
+  const unsigned QQ = (unsigned)(Q * nc);  // units of a block
+  const U* blocks = reinterpret_cast<const U*>(fac) + (size_t)pos * 9 * QQ;
+  // per node kUsed vectors of Qc values and the sums of its threads
+  T* v = reinterpret_cast<T*>(smem_raw) + (size_t)nd * (kUsed * Qc);
+  T* sums = reinterpret_cast<T*>(smem_raw) + (size_t)npc * (kUsed * Qc) + (size_t)nd * stride;
+  const U* mine0 = blocks + t;  // (t = g * Q + r: this thread's first unit of a block)
+  U buf[B];
 #pragma unroll
-  for (int sl = 0; sl < 9; ++sl) {
-    if (!fg_slot_used(c, sl, UPPER)) continue;
+  for (int b = 0; b < B; ++b) {
+    buf[b] = U{};
+    if (kUsed > 0 && b < mine) buf[b] = __ldg(mine0 + (unsigned)(fg_slot<C, UPPER>(0) * QQ + b * stride));
+  }
+  pdl_wait();
+  if (done != nullptr && *done) return;
+#pragma unroll
+  for (int k = 0; k < kUsed; ++k) {
     // a neighbour outside the mesh has a zero block and a zero vector: its clamped stand-in may
     // be a node this sweep has not written yet (the node itself at an even-sized mesh's edge)
-    const int nx = x + sl % 3 - 1, ny = y + sl / 3 - 1;
-    const bool inside = nx >= 0 && ny >= 0 && nx < m && ny < m;
-    const int jx = min(max(nx, 0), m - 1), jy = min(max(ny, 0), m - 1);
-    const T* src = Y + ((size_t)jx + (size_t)m * jy) * P + f0;
-    for (int t = r; t < Qc; t += G) v[k * Qc + t] = t < Q && inside ? src[t] : T(0);
-    ++k;
-  }
-  T acc = T(0);
-  if (!UPPER && r < Q)
-    acc = R[(size_t)i * P + f0 + r] - (sub != nullptr ? sub[(size_t)i * P + f0 + r] : T(0));
-  __syncthreads();
-  if (r < Q) {
-    unsigned used = 0;
-#pragma unroll
-    for (int sl = 0; sl < 9; ++sl) used |= fg_slot_used(c, sl, UPPER) ? 1u << sl : 0u;
-    // slot sl's vector is the k-th staged one, k = the used slots before it
-    if (UPPER)  // the diagonal first
-      acc = fg_block_row_dot<T, TV>(blocks + 4 * QQ, Q, r, v + (size_t)__popc(used & 15u) * Qc);
-#pragma unroll 1
-    for (int sl = 0; sl < 9; ++sl) {
-      if (sl == 4 || !(used >> sl & 1u)) continue;
-      acc -= fg_block_row_dot<T, TV>(blocks + sl * QQ, Q, r,
-                                     v + (size_t)__popc(used & ((1u << sl) - 1u)) * Qc);
+    constexpr auto slot = [](int kk) { return fg_slot<C, UPPER>(kk); };
+    const int sl = slot(k);
+    const int jx = x + sl % 3 - 1, jy = y + sl / 3 - 1;
+    const bool inside = jx >= 0 && jy >= 0 && jx < m && jy < m;
+    const T* src = Y + (inside ? ((size_t)jx + (size_t)m * jy) * P + f0 : 0);
+    for (int a = t; live && a < Qc; a += stride) {
+      const T val = a < Q && inside ? src[a] : T(0);
+      v[k * Qc + a] = sl == 4 ? val : -val;
     }
   }
-  if (live && r < Q) Y[(size_t)i * P + f0 + r] = acc;
+  T rhs = T(0);
+  if (!UPPER && live && t < Q)
+    rhs = R[(size_t)i * P + f0 + t] - (sub != nullptr ? sub[(size_t)i * P + f0 + t] : T(0));
+  __syncthreads();
+  T s0 = T(0), s1 = T(0), s2 = T(0), s3 = T(0);
+#pragma unroll
+  for (int k = 0; k < kUsed; ++k) {
+    const T* vv = v + k * Qc + (fg_quads<TV>() ? 4 : 1) * g;
+    for (int ch = 0; ch < nch; ++ch) {
+      // the batch after this one: in this block, or the first of the next used slot's
+      const bool same = ch + 1 < nch;
+      const int w0 = ch * B, wn = same ? w0 + B : 0;
+      const int lim = same || k + 1 < kUsed ? mine - wn : 0;
+      const unsigned next = (same ? fg_slot<C, UPPER>(k) : fg_slot<C, UPPER>(k + 1)) * QQ + wn * stride;
+#pragma unroll
+      for (int b = 0; b < B; ++b) {
+        if (w0 + b < mine) {
+          const int o = (w0 + b) * groups;
+          if constexpr (fg_quads<TV>()) {
+            const float2 u0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&buf[b].x));
+            const float2 u1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&buf[b].y));
+            const float4 x4 = *reinterpret_cast<const float4*>(vv + 4 * o);
+            s0 += u0.x * x4.x;
+            s1 += u0.y * x4.y;
+            s2 += u1.x * x4.z;
+            s3 += u1.y * x4.w;
+          } else {
+            (b & 1 ? s1 : s0) += (T)buf[b] * vv[o];
+          }
+        }
+        if (b < lim) buf[b] = __ldg(mine0 + (next + b * stride));
+      }
+    }
+  }
+  if (live) sums[t] = (s0 + s1) + (s2 + s3);
+  __syncthreads();
+  if (live && t < Q) {
+    T acc = rhs;
+    for (int gg = 0; gg < groups; ++gg) acc += sums[gg * Q + t];
+    Y[(size_t)i * P + f0 + t] = acc;
+  }
+}
+
+// Launch of colour c's phase.
+template <typename T, typename TV, bool UPPER>
+int launch_fg_phase(const System& s, int Q, int f0, int c, const TV* fac, const T* R, const T* sub,
+                    T* Y, cudaStream_t st, const int* done) {
+  const int cnt = s.cstart_h[c + 1] - s.cstart_h[c];
+  if (cnt <= 0) return SG_OK;
+  // groups: so many that a colour has about 1000 threads for every SM, each with a column at least
+  const int nc = fg_units<TV>(Q);
+  const long long wide = (1024 * 152LL + (long long)cnt * Q - 1) / ((long long)cnt * Q);
+  const int groups = (int)std::max(1LL, std::min<long long>(wide, std::min(nc, kFgThreads / Q)));
+  const int npc = std::max(1, std::min(cnt, kFgThreads / (groups * Q)));
+  // loads in flight per thread: 8, or 12 where a thread has more columns (n = 256, Q = 84 BF16:
+  // 1.39 ms; with 8 1.77, with 16 1.59, with 24, which leaves two CTAs per SM, 1.77); in FP64 8
+  constexpr int kB = sizeof(T) == 8 ? 8 : 12;
+  const bool deep = (nc + groups - 1) / groups > 8;
+  const int threads = (npc * groups * Q + 31) / 32 * 32;
+  int used = 0;
+  for (int sl = 0; sl < 9; ++sl) used += fg_slot_used(c, sl, UPPER);
+  const size_t smem = sizeof(T) * npc * ((size_t)used * fg_qc(Q) + (size_t)groups * Q);
+  TimeScope ts(s.timer, K_ILU_SOLVE, st);
+  auto go = [&](auto kern) {
+    SG_TRY(ensure_smem((const void*)kern, smem));
+    return launch_pdl(kern, dim3((cnt + npc - 1) / npc), dim3(threads), smem, st, s.pat.m, s.P, Q, f0,
+                      groups, npc, cnt, (const int*)s.cstart.p, fac, R, sub, Y, done);
+  };
+  int rc;
+  switch (c) {
+    case 0: rc = deep ? go(fg_phase_kernel<T, TV, UPPER, 0, kB>) : go(fg_phase_kernel<T, TV, UPPER, 0, 8>); break;
+    case 1: rc = deep ? go(fg_phase_kernel<T, TV, UPPER, 1, kB>) : go(fg_phase_kernel<T, TV, UPPER, 1, 8>); break;
+    case 2: rc = deep ? go(fg_phase_kernel<T, TV, UPPER, 2, kB>) : go(fg_phase_kernel<T, TV, UPPER, 2, 8>); break;
+    default: rc = deep ? go(fg_phase_kernel<T, TV, UPPER, 3, kB>) : go(fg_phase_kernel<T, TV, UPPER, 3, 8>); break;
+  }
+  return rc;
 }
 
 // tmp = D with the fields >= f0 set to zero (the earlier splits' solution).
 template <typename T>
 __global__ void fg_mask_kernel(size_t N, int P, int f0, const T* __restrict__ D, T* __restrict__ tmp,
                                const int* __restrict__ done) {
+  pdl_trigger();
+  pdl_wait();
   if (done != nullptr && *done) return;
   for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < N * P;
        t += (size_t)gridDim.x * blockDim.x)
@@ -602,8 +670,8 @@ int fg_apply(System& s, const T* R, T* D, cudaStream_t st, const int* done) {
     const T* sub = nullptr;
     if (si > 0) {  // Eq. P_group: subtract sum_{t < s} K_st z_t, from K applied to z masked
       TimeScope ts(s.timer, K_OTHER, st);
-      fg_mask_kernel<T><<<1216, 256, 0, st>>>((size_t)s.N, s.P, sp.f0, D, B::tmp(s), done);
-      SG_TRY(check_launch("fg_mask"));
+      SG_TRY(launch_pdl(fg_mask_kernel<T>, dim3(1216), dim3(256), 0, st, (size_t)s.N, s.P, sp.f0,
+                        (const T*)D, B::tmp(s), done));
       if (sizeof(T) == 8)
         SG_TRY(launch_matvec_f64(s, (const double*)B::tmp(s), (double*)B::tmp2(s), 1.0, nullptr,
                                  0.0, st, done));
@@ -612,34 +680,17 @@ int fg_apply(System& s, const T* R, T* D, cudaStream_t st, const int* done) {
                                  0.0f, st, done));
       sub = B::tmp2(s);
     }
-    const int G = fg_lanes(Q), nthr = fg_cta_threads(Q), npc = nthr / G;
-    const size_t smem = sizeof(T) * (size_t)npc * 9 * fg_qc(Q);
     for (int c = 0; c < 4; ++c) {
-      const int cnt = s.cstart_h[c + 1] - s.cstart_h[c];
-      if (cnt <= 0) continue;
-      TimeScope ts(s.timer, K_ILU_SOLVE, st);
-      const int grid = (cnt + npc - 1) / npc;
       if (fac16 != nullptr)
-        fg_phase_kernel<T, __nv_bfloat16, false><<<grid, nthr, smem, st>>>(
-            s.pat.m, s.P, Q, sp.f0, c, s.cstart.p, fac16, R, sub, D, done);
+        SG_TRY((launch_fg_phase<T, __nv_bfloat16, false>(s, Q, sp.f0, c, fac16, R, sub, D, st, done)));
       else
-        fg_phase_kernel<T, T, false><<<grid, nthr, smem, st>>>(s.pat.m, s.P, Q, sp.f0, c,
-                                                              s.cstart.p, fac, R, sub, D, done);
-      SG_TRY(check_launch("fg_phase (forward)"));
+        SG_TRY((launch_fg_phase<T, T, false>(s, Q, sp.f0, c, fac, R, sub, D, st, done)));
     }
     for (int c = 3; c >= 0; --c) {
-      const int cnt = s.cstart_h[c + 1] - s.cstart_h[c];
-      if (cnt <= 0) continue;
-      TimeScope ts(s.timer, K_ILU_SOLVE, st);
-      const int grid = (cnt + npc - 1) / npc;
       if (fac16 != nullptr)
-        fg_phase_kernel<T, __nv_bfloat16, true><<<grid, nthr, smem, st>>>(
-            s.pat.m, s.P, Q, sp.f0, c, s.cstart.p, fac16, nullptr, nullptr, D, done);
+        SG_TRY((launch_fg_phase<T, __nv_bfloat16, true>(s, Q, sp.f0, c, fac16, nullptr, nullptr, D, st, done)));
       else
-        fg_phase_kernel<T, T, true><<<grid, nthr, smem, st>>>(s.pat.m, s.P, Q, sp.f0, c,
-                                                             s.cstart.p, fac, nullptr, nullptr, D,
-                                                             done);
-      SG_TRY(check_launch("fg_phase (backward)"));
+        SG_TRY((launch_fg_phase<T, T, true>(s, Q, sp.f0, c, fac, nullptr, nullptr, D, st, done)));
     }
   }
   return SG_OK;

@@ -180,6 +180,8 @@ __global__ void __launch_bounds__(kRedThreads) cgs_dots_kernel(
     size_t n, const double* __restrict__ V, int nv, double* __restrict__ w,
     const float* __restrict__ w32, double* __restrict__ partial, unsigned int* ticket,
     double* __restrict__ h, const int* __restrict__ done) {
+  pdl_trigger();
+  pdl_wait();
   if (*done) return;
   __shared__ double sh[kRedThreads / 32][kLT];
   if (w32 != nullptr)
@@ -196,6 +198,8 @@ __global__ void __launch_bounds__(kRedThreads) cgs_update_dots_kernel(
     size_t n, const double* __restrict__ V, int nv, double* __restrict__ w,
     const double* __restrict__ h1, double* __restrict__ partial, unsigned int* ticket,
     double* __restrict__ h2, const int* __restrict__ done) {
+  pdl_trigger();
+  pdl_wait();
   if (*done) return;
   __shared__ double sh[kRedThreads / 32][kLT];
   __shared__ double hs[kMaxBasis];
@@ -222,6 +226,8 @@ __global__ void __launch_bounds__(kRedThreads) cgs_update_norm_kernel(
     unsigned int* ticket, double* __restrict__ Hs, int ldh, double* __restrict__ cs,
     double* __restrict__ sn, double* __restrict__ g, double* __restrict__ state,
     int* __restrict__ flags, int last_col) {
+  pdl_trigger();
+  pdl_wait();
   if (flags[0]) return;
   __shared__ double sh[32];
   __shared__ double hs[kMaxBasis], c_s[kMaxBasis], s_s[kMaxBasis], cn[kMaxBasis];
@@ -304,6 +310,8 @@ __global__ void __launch_bounds__(kStepThreads)
   double* sums = s_s + nv;       // shares' sums (step_sums entries), then the Givens scratch
   __shared__ double red[32], scal[2];
   __shared__ int skip;
+  pdl_trigger();
+  pdl_wait();
   if (threadIdx.x == 0) skip = flags[0];
   // (the flag changes only in this kernel's last phase, after a cluster barrier)
   __syncthreads();
@@ -458,6 +466,8 @@ int step_ctas() {
 // with ``v32`` also its FP32 copy, the next step's preconditioner operand
 __global__ void scale_kernel(size_t n, double* __restrict__ v, float* __restrict__ v32,
                              const double* __restrict__ state, const int* __restrict__ flags) {
+  pdl_trigger();
+  pdl_wait();
   if (flags[0]) return;
   double sc = state[3];
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -634,12 +644,14 @@ int k_arnoldi(System& s, size_t n, int j, int last_col, const float* w32, cudaSt
     cfg.blockDim = dim3(kStepThreads, 1, 1);
     cfg.dynamicSmemBytes = stage ? head + slices : head;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)ctas;
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     TimeScope ts(s.timer, K_ARNOLDI, st);
     SG_CUDA(cudaLaunchKernelEx(&cfg, arnoldi_cluster_kernel, (int)n, (const double*)s.V.p, nv, w, w32,
                                s.Hs.p, s.m + 1, s.cs.p, s.sn.p, s.g.p, s.scal.p, s.flags.p, last_col,
@@ -649,28 +661,26 @@ int k_arnoldi(System& s, size_t n, int j, int last_col, const float* w32, cudaSt
   const int grid = red_grid(n);
   {
     TimeScope ts(s.timer, K_ARNOLDI, st);
-    cgs_dots_kernel<<<grid, kRedThreads, 0, st>>>(n, s.V.p, nv, w, w32, s.red.p, s.ticket.p, h1,
-                                                  s.flags.p);
+    SG_TRY(launch_pdl(cgs_dots_kernel, dim3(grid), dim3(kRedThreads), 0, st, n, (const double*)s.V.p, nv,
+                      w, w32, s.red.p, s.ticket.p, h1, (const int*)s.flags.p));
   }
-  SG_TRY(check_launch("cgs_dots"));
   {
     TimeScope ts(s.timer, K_ARNOLDI, st);
-    cgs_update_dots_kernel<<<grid, kRedThreads, 0, st>>>(n, s.V.p, nv, w, h1, s.red.p, s.ticket.p,
-                                                         h2, s.flags.p);
+    SG_TRY(launch_pdl(cgs_update_dots_kernel, dim3(grid), dim3(kRedThreads), 0, st, n,
+                      (const double*)s.V.p, nv, w, (const double*)h1, s.red.p, s.ticket.p, h2,
+                      (const int*)s.flags.p));
   }
-  SG_TRY(check_launch("cgs_update_dots"));
   {
     TimeScope ts(s.timer, K_ARNOLDI, st);
-    cgs_update_norm_kernel<<<grid, kRedThreads, 0, st>>>(
-        n, s.V.p, nv, w, h1, h2, s.red.p, s.ticket.p, s.Hs.p, s.m + 1, s.cs.p, s.sn.p, s.g.p,
-        s.scal.p, s.flags.p, last_col);
+    SG_TRY(launch_pdl(cgs_update_norm_kernel, dim3(grid), dim3(kRedThreads), 0, st, n,
+                      (const double*)s.V.p, nv, w, (const double*)h1, (const double*)h2, s.red.p,
+                      s.ticket.p, s.Hs.p, s.m + 1, s.cs.p, s.sn.p, s.g.p, s.scal.p, s.flags.p, last_col));
   }
-  SG_TRY(check_launch("cgs_update_norm"));
   {
     TimeScope ts(s.timer, K_ARNOLDI, st);
-    scale_kernel<<<kRedBlocks, kRedThreads, 0, st>>>(n, w, s.mv32a.p, s.scal.p, s.flags.p);
+    return launch_pdl(scale_kernel, dim3(kRedBlocks), dim3(kRedThreads), 0, st, n, w, s.mv32a.p,
+                      (const double*)s.scal.p, (const int*)s.flags.p);
   }
-  return check_launch("scale");
 }
 
 int k_finish_cycle(System& s, size_t n, double* x, bool z32, cudaStream_t st) {

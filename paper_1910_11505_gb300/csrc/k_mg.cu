@@ -23,6 +23,8 @@ namespace {
 template <typename T>
 __global__ void restrict_kernel(const T* __restrict__ rf, T* __restrict__ bc, int nc, int P,
                                 const int* __restrict__ done) {
+  pdl_trigger();
+  pdl_wait();
   if (done != nullptr && *done) return;
   const int mc = nc + 1, mf = 2 * nc + 1;
   const long long total = (long long)mc * mc * P;
@@ -51,6 +53,8 @@ __global__ void restrict_kernel(const T* __restrict__ rf, T* __restrict__ bc, in
 template <typename T>
 __global__ void prolong_add_kernel(const T* __restrict__ uc, T* __restrict__ uf, int nc, int P,
                                    const int* __restrict__ done) {
+  pdl_trigger();
+  pdl_wait();
   if (done != nullptr && *done) return;
   const int mc = nc + 1, mf = 2 * nc + 1;
   const long long total = (long long)mf * mf * P;
@@ -78,6 +82,8 @@ template <typename T>
 __global__ void coarse_solve_kernel(const T* __restrict__ inv, const int* __restrict__ nodes,
                                     int nint, int N, int P, const T* __restrict__ b,
                                     T* __restrict__ u, const int* __restrict__ done) {
+  pdl_trigger();
+  pdl_wait();
   if (done != nullptr && *done) return;
   const int dim = nint * P;
   const int lane = threadIdx.x & 31;
@@ -187,8 +193,8 @@ template <typename T>
 int launch_restrict(const T* rf, T* bc, int nc, int P, cudaStream_t st, const int* done,
                     Timer* timer) {
   TimeScope ts(timer, K_OTHER, st);
-  restrict_kernel<T><<<grid_for((long long)(nc + 1) * (nc + 1) * P), 256, 0, st>>>(rf, bc, nc, P, done);
-  return check_launch("mg_restrict");
+  return launch_pdl(restrict_kernel<T>, dim3(grid_for((long long)(nc + 1) * (nc + 1) * P)), dim3(256), 0,
+                    st, rf, bc, nc, P, done);
 }
 
 template <typename T>
@@ -196,8 +202,8 @@ int launch_prolong_add(const T* uc, T* uf, int nc, int P, cudaStream_t st, const
                        Timer* timer) {
   TimeScope ts(timer, K_OTHER, st);
   const long long mf = 2 * nc + 1;
-  prolong_add_kernel<T><<<grid_for(mf * mf * P), 256, 0, st>>>(uc, uf, nc, P, done);
-  return check_launch("mg_prolong");
+  return launch_pdl(prolong_add_kernel<T>, dim3(grid_for(mf * mf * P)), dim3(256), 0, st, uc, uf, nc, P,
+                    done);
 }
 
 template <typename T>
@@ -209,8 +215,8 @@ int launch_coarse_solve(const System& c, const T* b, T* u, cudaStream_t st, cons
   TimeScope ts(c.timer, K_OTHER, st);
   const int dim = c.mg_nint * c.P;
   const int grid = std::max(1, std::min(152 * 4, (dim + 7) / 8));
-  coarse_solve_kernel<T><<<grid, 256, 0, st>>>(inv, c.mg_nodes.p, c.mg_nint, c.N, c.P, b, u, done);
-  return check_launch("mg_coarse_solve");
+  return launch_pdl(coarse_solve_kernel<T>, dim3(grid), dim3(256), 0, st, inv, (const int*)c.mg_nodes.p,
+                    c.mg_nint, c.N, c.P, b, u, done);
 }
 
 template int launch_restrict<double>(const double*, double*, int, int, cudaStream_t, const int*, Timer*);

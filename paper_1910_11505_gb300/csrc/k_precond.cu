@@ -15,6 +15,8 @@
 // path.  The off-diagonal coupling of the Gauss-Seidel sweep, sum_{b<a} K_ab z_b, is subtracted
 // from the later columns of rhs_t after each block b by a grid-wide kernel:
 // T[k] = sum_e A[e,k] z_b[j_e] once per (row, k), then rhs_t[a] -= G_k[a,b] T[k] for a > b.
+#include <algorithm>
+
 #include "sg_internal.h"
 
 namespace sg {
@@ -715,6 +717,8 @@ __global__ void __launch_bounds__(256) fs_next_kernel(
 template <typename T>
 __global__ void axpy_kernel(size_t n, const T* __restrict__ x, T* __restrict__ y,
                             const int* __restrict__ done) {
+  pdl_trigger();
+  pdl_wait();
   if (done != nullptr && *done) return;
   for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n;
        t += (size_t)gridDim.x * blockDim.x)
@@ -956,8 +960,8 @@ int matvec_t<float>(const System& s, const float* X, float* Y, float alpha, cons
 template <typename T>
 int launch_axpy(System& s, size_t n, const T* x, T* y, cudaStream_t st, const int* done) {
   TimeScope ts(s.timer, K_OTHER, st);
-  axpy_kernel<T><<<1216, 256, 0, st>>>(n, x, y, done);
-  return check_launch("axpy");
+  const int grid = (int)std::max<size_t>(1, std::min<size_t>(1216, (n + 255) / 256));
+  return launch_pdl(axpy_kernel<T>, dim3(grid), dim3(256), 0, st, n, x, y, done);
 }
 
 // Multigrid vectors of one level in the working precision.

@@ -100,6 +100,29 @@ __device__ __forceinline__ void l2_prefetch(const void* base, size_t bytes, int 
   }
 }
 
+// Programmatic dependent launch.  A kernel launched by launch_pdl may start while the kernel before
+// it on the stream still runs; until pdl_wait() it may only read what no queued kernel writes
+// (factors, assembled blocks, tables) and write nothing.  pdl_trigger() lets the next kernel start
+// once every CTA of this one has passed it.  Both are no-ops in an ordinary launch.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... KA, typename... A>
+int launch_pdl(void (*kern)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  SG_CUDA(cudaLaunchKernelEx(&cfg, kern, static_cast<KA>(args)...));
+  return check_launch("kernel");
+}
+
 // mbarrier and 1-D bulk-copy (cp.async.bulk) helpers.  Every wait is bounded: after kWaitLimit
 // polls it gives up and the caller takes its error path.
 constexpr long long kWaitLimit = 1LL << 22;
