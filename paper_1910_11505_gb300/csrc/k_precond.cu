@@ -929,6 +929,9 @@ int apply_block(System& s, const T* R, T* D, cudaStream_t st, const int* done) {
   switch (s.pc_fac) {
     case SG_PC_MEAN:
     case SG_PC_FS_JACOBI:
+      if constexpr (sizeof(T) == 4)
+        if (s.wave_v.p != nullptr)
+          return launch_wave_solve(s, s.pc_fac == SG_PC_FS_JACOBI ? 1 : 0, R, D, st, done);
       SG_TRY(launch_columns<T>(s, R, B::rhs_t(s), st, done));
       return launch_block_solve<T>(s, 0, s.P, s.pc_fac == SG_PC_FS_JACOBI ? 1 : 0,
                                    B::rhs_t(s), D, st, done);

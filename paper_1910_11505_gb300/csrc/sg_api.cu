@@ -521,7 +521,7 @@ static void free_system(System* s) {
                         &s->tmp2, &s->tri_w, &s->V, &s->Z, &s->Hs, &s->cs, &s->sn, &s->g, &s->y,
                         &s->scal, &s->red, &s->rvec};
   for (auto* b : db) b->release();
-  DBuf<float>* fb[] = {&s->stack_f32, &s->stack_km32, &s->ent_g_f32, &s->lu9_f32, &s->blk_f32, &s->gs_eg_f32, &s->gsn_eg_f32, &s->gsn_cs32, &s->gsn_corr32,
+  DBuf<float>* fb[] = {&s->stack_f32, &s->stack_km32, &s->ent_g_f32, &s->lu9_f32, &s->wave_low, &s->wave_up, &s->wave_v, &s->blk_f32, &s->gs_eg_f32, &s->gsn_eg_f32, &s->gsn_cs32, &s->gsn_corr32,
                        &s->rhs_t32, &s->tmp32, &s->tmp232, &s->tri_w32, &s->V32, &s->Z32,
                        &s->mv32a, &s->mv32b};
   for (auto* b : fb) b->release();
@@ -649,6 +649,7 @@ static int setup_system(System& s, cudaStream_t st, bool krylov = true) {
     } else {
       SG_TRY(launch_ilu0(s, st));
       SG_TRY(launch_lu9(s, st));
+      if (lowp && s.pc_fac != SG_PC_FS_GS && p.inner_iters == 1) SG_TRY(wave_setup(s, st));
     }
     if (lowp) {
       SG_TRY(s.lu9_f32.alloc(s.lu9.n));
@@ -1073,7 +1074,7 @@ int sg_setup(const sg_params* prm, int nsys, void* stream, sg_handle** out) {
   for (int i = 0; i < nsys; ++i) SG_TRY(validate(prm[i]));
   cudaStream_t st = (cudaStream_t)stream;
   // where the device's memory does not hold all systems, once more without the block-stencil
-  // operators, whose memory the other forms do not need
+  // operators and the warps' factor streams, whose memory the other forms do not need
   for (const bool lean : {false, true}) {
     sg_handle* h = new sg_handle();
     cudaGetDevice(&h->device);
@@ -1086,7 +1087,7 @@ int sg_setup(const sg_params* prm, int nsys, void* stream, sg_handle** out) {
       s->lean = lean;
       h->sys.push_back(s);
       rc = setup_system(*s, st);
-      blocks = blocks || s->block64.ready || s->block32.ready;
+      blocks = blocks || s->block64.ready || s->block32.ready || s->wave_low.p != nullptr;
       if (rc != SG_OK) fail(rc, "system " + std::to_string(i) + ": " + std::string(g_last_error));
     }
     if (rc == SG_OK) rc = make_pool(h, st);

@@ -339,6 +339,8 @@ struct System {
   DBuf<float> blk_f32;         // FP32 copy for the mixed inner solver
   DBuf<double> lu9;            // nfac x 9 x N level-major slot layout of the factors
   DBuf<float> lu9_f32;
+  // natural order, mixed mean-based and Jacobi forms (k_ilu_wave.cu): factor streams, columns
+  DBuf<float> wave_low, wave_up, wave_v;
   DBuf<int> lev9_off;          // start of each wavefront level in level-major order
   DBuf<int> cstart;            // four-colour ordering: start of each colour (5 offsets)
   int nlev9 = 0;
@@ -457,6 +459,11 @@ int launch_color_solve(System& s, int a0, int ncols, int fac_per_col, const T* l
 // BF16-rounded stiffness values when the sweep couples in BF16), from the FP64 k-major stack.
 int launch_color_coupling(System& s, cudaStream_t st);
 int launch_lu9(System& s, cudaStream_t st);
+// Natural-order solves of all columns by warps in FP32 (k_ilu_wave.cu): setup (wave_v stays empty
+// where they do not apply) and one application.
+int wave_setup(System& s, cudaStream_t st);
+int launch_wave_solve(System& s, int fac_per_col, const float* R, float* Z, cudaStream_t st,
+                      const int* done);
 int launch_cast_f32(const double* src, float* dst, size_t n, cudaStream_t st);
 int launch_cast_bf16(const double* src, __nv_bfloat16* dst, size_t n, cudaStream_t st);
 int launch_cast_f64(const float* src, double* dst, size_t n, cudaStream_t st);
