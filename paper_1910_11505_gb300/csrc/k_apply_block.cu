@@ -103,6 +103,9 @@ __global__ void __launch_bounds__((kBlockMaxWarps + 1) * 32) block_edge_kernel(
   const int slot_mask = g.slots - 1, slot_log = __ffs(g.slots) - 1;
   const int row0 = m + 1, nrows = g.N - 2 * (m + 1);
   const int nitems = g.ntiles_row * kBlockEdges;
+  // The next kernel's CTAs come in with a CTA's last item: earlier they would only take room from
+  // the items' (256 x 256 FP32: 773 us with the trigger here for all, 752 us without).
+  if (nitems <= (int)gridDim.x) pdl_trigger();
   for (int i = tid; i < g.rounds * nb; i += blockDim.x) tab[i] = table[i];
   for (int i = tid; i < g.ntile; i += blockDim.x) kinds[i] = tkind[i];
   if (tid == 0) {
@@ -191,6 +194,7 @@ __global__ void __launch_bounds__((kBlockMaxWarps + 1) * 32) block_edge_kernel(
   };
   if (sizeof(T) == 4 && (int)blockIdx.x < nitems) fetch(blockIdx.x);
   for (int it = blockIdx.x; it < nitems; it += gridDim.x, base += (unsigned)g.ntile) {
+    if (nitems > (int)gridDim.x && it + (int)gridDim.x >= nitems) pdl_trigger();
     const int t = it / kBlockEdges, e = it - t * kBlockEdges;
     if (sizeof(T) == 8) fetch(it);
 #pragma unroll
@@ -262,8 +266,6 @@ __global__ void __launch_bounds__((kBlockMaxWarps + 1) * 32) block_edge_kernel(
         o[q] = D[b * kBLd + r];
       }
     }
-    // (the next kernel's CTAs do not share the SMs with more than the last items)
-    if (it + (int)gridDim.x >= nitems) pdl_trigger();
   }
 }
 

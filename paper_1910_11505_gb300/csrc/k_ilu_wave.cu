@@ -20,7 +20,7 @@
 // Bound: the dependent chain of a step (a shuffle and two multiply-adds) and its instructions.
 // FP64 keeps the barrier kernels: four or five multiply-adds of 65 cycles each on one
 // sub-partition would bound a step here.  One application by 84 columns on one GB300, barrier kernels
-// -> here: 128 x 128 150 -> 74 us, 256 x 256 571 -> 152 us.
+// -> here: 128 x 128 150 -> 74 us, 256 x 256 571 -> 123 us.
 #include <algorithm>
 
 #include "sg_internal.h"
@@ -108,7 +108,7 @@ __device__ __forceinline__ void wave_sweep(float* val, const float* ring, unsign
   };
   auto wait_block = [&](int b) {
     const unsigned u = use0 + b;
-    if (!*vfail && !mbar_wait_bounded(&full[u % kWaveSlots], (u / kWaveSlots) & 1u)) *vfail = 1;
+    mbar_wait_or_fail(&full[u % kWaveSlots], (u / kWaveSlots) & 1u, vfail);
   };
   wait_block(0);
   take(0, 0, f[0], dinv[0], wv[0]);
@@ -116,7 +116,7 @@ __device__ __forceinline__ void wave_sweep(float* val, const float* ring, unsign
   for (int b = 0; b < nblk; ++b) {
     // this block's steps read ahead to step 8 b + 71 of the line before
     if (!first) {
-      if (!*vfail && !mbar_wait_bounded(&done_prev[min(b + 8, nblk - 1)], UPPER ? 1u : 0u)) *vfail = 1;
+      mbar_wait_or_fail(&done_prev[min(b + 8, nblk - 1)], UPPER ? 1u : 0u, vfail);
       if (b == 0) {  // the line before at the next and at this node of the first step
         bn = bnd_prev[63];
         if (lane == in_lane) up2 = bnd_prev[62];

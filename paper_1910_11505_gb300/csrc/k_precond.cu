@@ -776,6 +776,8 @@ int launch_block_solve(System& s, int a0, int ncols, int fac_per_col, const T* R
   using B = PcBufs<T>;
   if (s.prm.ilu_order == SG_ILU_COLOR4)
     return launch_color_solve<T>(s, a0, ncols, fac_per_col, B::lu9(s), const_cast<T*>(Rt), Z, st, done);
+  if constexpr (sizeof(T) == 8)
+    if (s.line_fac.p != nullptr) return launch_lines_solve(s, a0, ncols, fac_per_col, Rt, Z, st, done);
   const int wc = s.tri_wc;
   const bool full = B::full(s);
   const int nthreads = 2 * wc + (full ? 32 : tri_staging_threads(wc));

@@ -518,7 +518,7 @@ static void free_system(System* s) {
   for (auto* b : {&s->fg_tmp, &s->fg_tmp2}) b->release();
   for (auto* b : {&s->fg_tmp32, &s->fg_tmp232}) b->release();
   DBuf<double>* db[] = {&s->stack, &s->stack_km, &s->ent_g, &s->blk, &s->fac, &s->lu9, &s->gs_eg, &s->gsn_eg, &s->gsn_cs, &s->gsn_corr, &s->rhs_t, &s->tmp,
-                        &s->tmp2, &s->tri_w, &s->V, &s->Z, &s->Hs, &s->cs, &s->sn, &s->g, &s->y,
+                        &s->tmp2, &s->line_fac, &s->line_dinv, &s->tri_w, &s->V, &s->Z, &s->Hs, &s->cs, &s->sn, &s->g, &s->y,
                         &s->scal, &s->red, &s->rvec};
   for (auto* b : db) b->release();
   DBuf<float>* fb[] = {&s->stack_f32, &s->stack_km32, &s->ent_g_f32, &s->lu9_f32, &s->wave_low, &s->wave_up, &s->wave_v, &s->blk_f32, &s->gs_eg_f32, &s->gsn_eg_f32, &s->gsn_cs32, &s->gsn_corr32,
@@ -650,6 +650,7 @@ static int setup_system(System& s, cudaStream_t st, bool krylov = true) {
       SG_TRY(launch_ilu0(s, st));
       SG_TRY(launch_lu9(s, st));
       if (lowp && s.pc_fac != SG_PC_FS_GS && p.inner_iters == 1) SG_TRY(wave_setup(s, st));
+      if (!lowp && p.inner_iters == 1) SG_TRY(lines_setup(s, st));
     }
     if (lowp) {
       SG_TRY(s.lu9_f32.alloc(s.lu9.n));
@@ -1087,7 +1088,8 @@ int sg_setup(const sg_params* prm, int nsys, void* stream, sg_handle** out) {
       s->lean = lean;
       h->sys.push_back(s);
       rc = setup_system(*s, st);
-      blocks = blocks || s->block64.ready || s->block32.ready || s->wave_low.p != nullptr;
+      blocks = blocks || s->block64.ready || s->block32.ready || s->wave_low.p != nullptr ||
+               s->line_fac.p != nullptr;
       if (rc != SG_OK) fail(rc, "system " + std::to_string(i) + ": " + std::string(g_last_error));
     }
     if (rc == SG_OK) rc = make_pool(h, st);

@@ -162,6 +162,13 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsig
   return false;
 }
 
+// The same for warps that share a failure flag: once one gave up, the others wait no more.
+__device__ __forceinline__ void mbar_wait_or_fail(unsigned long long* bar, unsigned parity,
+                                                  volatile int* fail) {
+  if (mbar_try_wait(bar, parity)) return;
+  if (!*fail && !mbar_wait_bounded(bar, parity)) *fail = 1;
+}
+
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned bytes,
                                          unsigned long long* bar) {
   asm volatile(
@@ -341,6 +348,8 @@ struct System {
   DBuf<float> lu9_f32;
   // natural order, mixed mean-based and Jacobi forms (k_ilu_wave.cu): factor streams, columns
   DBuf<float> wave_low, wave_up, wave_v;
+  // natural order, FP64 (k_ilu_lines.cu): factor streams, 1/u_ii by lines
+  DBuf<double> line_fac, line_dinv;
   DBuf<int> lev9_off;          // start of each wavefront level in level-major order
   DBuf<int> cstart;            // four-colour ordering: start of each colour (5 offsets)
   int nlev9 = 0;
@@ -464,6 +473,11 @@ int launch_lu9(System& s, cudaStream_t st);
 int wave_setup(System& s, cudaStream_t st);
 int launch_wave_solve(System& s, int fac_per_col, const float* R, float* Z, cudaStream_t st,
                       const int* done);
+// Natural-order solves by warps in FP64 (k_ilu_lines.cu): setup (line_fac stays empty where they do
+// not apply) and the solve of columns a0 .. a0 + ncols - 1 from Rt into Z.
+int lines_setup(System& s, cudaStream_t st);
+int launch_lines_solve(System& s, int a0, int ncols, int fac_per_col, const double* Rt, double* Z,
+                       cudaStream_t st, const int* done);
 int launch_cast_f32(const double* src, float* dst, size_t n, cudaStream_t st);
 int launch_cast_bf16(const double* src, __nv_bfloat16* dst, size_t n, cudaStream_t st);
 int launch_cast_f64(const float* src, double* dst, size_t n, cudaStream_t st);
