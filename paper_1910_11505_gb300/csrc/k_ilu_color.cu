@@ -8,6 +8,8 @@
 // (dy+1)*3 + (dx+1) for the neighbour at (x+dx, y+dy), absent neighbours 0): slots whose neighbour
 // has a lower colour hold the unit lower factor l_ij, slots of a higher colour hold u_ij / u_ii,
 // slot 4 holds 1 / u_ii.
+#include <algorithm>
+
 #include "sg_internal.h"
 
 namespace sg {
@@ -310,37 +312,32 @@ __device__ __forceinline__ void color_sweeps(int off, int stride, int m, int N, 
   }
 }
 
-// All eight phases of one column in one CTA, the column in shared memory (meshes whose column
-// fits): CTA b solves column a0 + b.  The solution goes to column a of Z and, contiguous, back
-// over column a of Rt (as the cluster kernel leaves it), where the coupling scatter reads it.
-// A single-column launch first prefetches the column's factors (and coupling stencil) into L2, so
-// only the first phase waits for HBM.
+// All eight phases of column a in one CTA, the column in shared memory (meshes whose column fits).
+// The solution goes to column a of Z (if any) and, contiguous, back over column a of Rt (as the
+// cluster kernel leaves it), where the coupling scatter reads it.  ``prefetch``: where the factors (and
+// the coupling stencil) do not fit beside the column, they are fetched into L2 first.
+//
+// stage >= 1: the factors (stage 2: also the coupling stencil) are copied into shared memory
+// after the column by one bulk copy each, issued before the kernel before this one has ended; a
+// copy takes the 16-byte-aligned range around its array (the arrays are padded for that) and
+// the phases index from the offset.  Should the bounded wait give up, the phases read the
+// arrays in global memory instead (same values).
 template <typename T>
-__global__ void __launch_bounds__(1024) color_cta_kernel(int m, int N, int ldN, int P, int a0,
-                                                        int fac_per_col, const int* __restrict__ cstart_g,
-                                                        const T* __restrict__ cfs,
-                                                        T* __restrict__ Rt, T* __restrict__ Z,
-                                                        const int* __restrict__ done,
-                                                        const T* __restrict__ cs, T* __restrict__ corr,
-                                                        int stage) {
-  if (done != nullptr && *done) return;
+__device__ __forceinline__ void color_cta_solve(int m, int N, int ldN, int P, int a, int fac_per_col,
+                                                const int* __restrict__ cstart_g,
+                                                const T* __restrict__ cfs, T* __restrict__ Rt,
+                                                T* __restrict__ Z, const int* __restrict__ done,
+                                                const T* __restrict__ cs, T* __restrict__ corr,
+                                                int stage, bool prefetch) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* w = reinterpret_cast<T*>(smem_raw);
   __shared__ int cstart[5];
-  const int a = a0 + blockIdx.x;
+  __shared__ unsigned long long bar;
   const T* cf = cfs + (size_t)(fac_per_col ? a : 0) * 9 * N;
   T* rhs = Rt + (size_t)a * ldN;
   const T* corr_in = (cs != nullptr && a > 0) ? corr : nullptr;
   const T* csn = (cs != nullptr && a + 1 < P) ? cs + (size_t)a * 9 * N : nullptr;
-  // stage >= 1: the factors (stage 2: also the coupling stencil) are copied into shared memory
-  // after the column by one bulk copy each, issued before the column load so the two overlap; a
-  // copy takes the 16-byte-aligned range around its array (the arrays are padded for that) and
-  // the phases index from the offset.  Should the bounded wait give up, the phases read the
-  // arrays in global memory instead (same values).
-  __shared__ unsigned long long bar;
   unsigned char* buf = smem_raw + sizeof(T) * (size_t)ldN;
-  const T* cf_s = nullptr;
-  const T* cs_s = nullptr;
   if (stage >= 1) {
     if (threadIdx.x == 0) {
       mbar_init(&bar, 1);
@@ -359,33 +356,74 @@ __global__ void __launch_bounds__(1024) color_cta_kernel(int m, int N, int ldN, 
       bulk_g2s(buf, reinterpret_cast<const void*>(lo_cf), n_cf, &bar);
       if (n_cs) bulk_g2s(buf + kColorSlotBuf(N, sizeof(T)), reinterpret_cast<const void*>(lo_cs), n_cs, &bar);
     }
-  } else if (gridDim.x == 1) {
+  } else if (prefetch) {
     l2_prefetch(cf, sizeof(T) * 9 * (size_t)N, 0, 1);
     if (csn != nullptr) l2_prefetch(csn, sizeof(T) * 9 * (size_t)N, 0, 1);
   }
   if (threadIdx.x < 5) cstart[threadIdx.x] = cstart_g[threadIdx.x];
-  for (int i = threadIdx.x; i < N; i += blockDim.x) w[i] = rhs[i];
+  pdl_wait();
+  const bool skip = done != nullptr && *done;
+  if (!skip)
+    for (int i = threadIdx.x; i < N; i += blockDim.x) w[i] = rhs[i];
   __syncthreads();
-  bool staged = false;
-  if (stage >= 1) {
-    staged = mbar_wait_bounded(&bar, 0);
-    if (staged) {
-      cf_s = reinterpret_cast<const T*>(buf + (reinterpret_cast<unsigned long long>(cf) & 15ull));
-      cf = cf_s;
-      if (stage >= 2 && csn != nullptr) {
-        cs_s = reinterpret_cast<const T*>(buf + kColorSlotBuf(N, sizeof(T)) +
-                                          (reinterpret_cast<unsigned long long>(csn) & 15ull));
-        csn = cs_s;
-      }
+  if (stage >= 1 && mbar_wait_bounded(&bar, 0)) {
+    cf = reinterpret_cast<const T*>(buf + (reinterpret_cast<unsigned long long>(cf) & 15ull));
+    if (stage >= 2 && csn != nullptr)
+      csn = reinterpret_cast<const T*>(buf + kColorSlotBuf(N, sizeof(T)) +
+                                       (reinterpret_cast<unsigned long long>(csn) & 15ull));
+    stage = 0;
+  }
+  if (!skip) {
+    color_sweeps<T, false>(threadIdx.x, blockDim.x, m, N, P, a, cstart, cf, w, corr_in, csn, corr,
+                           (T*)nullptr, []() { __syncthreads(); });
+    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+      if (Z != nullptr) Z[(size_t)i * P + a] = w[i];
+      rhs[i] = w[i];
     }
   }
-  color_sweeps<T, false>(threadIdx.x, blockDim.x, m, N, P, a, cstart, cf, w, corr_in, csn, corr,
-                         (T*)nullptr, []() { __syncthreads(); });
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    if (Z != nullptr) Z[(size_t)i * P + a] = w[i];
-    rhs[i] = w[i];
+  if (stage >= 1) mbar_wait_bounded(&bar, 0);  // no copy may land after the exit
+}
+
+// CTA b solves column a0 + b.
+template <typename T>
+__global__ void __launch_bounds__(1024) color_cta_kernel(int m, int N, int ldN, int P, int a0,
+                                                        int fac_per_col, const int* __restrict__ cstart_g,
+                                                        const T* __restrict__ cfs,
+                                                        T* __restrict__ Rt, T* __restrict__ Z,
+                                                        const int* __restrict__ done,
+                                                        const T* __restrict__ cs, T* __restrict__ corr,
+                                                        int stage) {
+  color_cta_solve<T>(m, N, ldN, P, a0 + (int)blockIdx.x, fac_per_col, cstart_g, cfs, Rt, Z, done, cs,
+                     corr, stage, gridDim.x == 1);
+}
+
+// One step of the Gauss-Seidel sweep: CTA 0 solves block a, the others subtract block a - 1's
+// coupling from the columns a + 1 ..  Both need only what the step before left (column a of Rt has
+// the couplings up to a - 2 then, and ``corr`` that of a - 1), so the steps follow one another on one
+// stream as programmatic launches: the next solve's CTA takes an idle SM at once and has its
+// factors in shared memory when this step ends.
+// Bound: the latency of nine dependent phases and of the hand-over between two launches.
+// Measured on one GB300: a V-cycle with 35 columns, FP32, 128 x 128 down to 4 x 4 (350 steps of this
+// kernel, 70 of the clusters) 6.50 -> 5.06 ms against a launch for each with the scatters on a second stream.
+template <typename T, typename TV>
+__global__ void __launch_bounds__(1024) color_gs_kernel(
+    int m, int N, int ldN, int P, int nnz, int a, const int* __restrict__ cstart_g,
+    const T* __restrict__ cfs, T* __restrict__ Rt, const int* __restrict__ done,
+    const T* __restrict__ cs, T* __restrict__ corr, int stage, const int* __restrict__ rowptr,
+    const int* __restrict__ col, const TV* __restrict__ stack_km, const int* __restrict__ kptr,
+    const int* __restrict__ klist, const int* __restrict__ eptr, const int* __restrict__ ek,
+    const T* __restrict__ eg) {
+  pdl_trigger();
+  if (blockIdx.x == 0) {
+    color_cta_solve<T>(m, N, ldN, P, a, 1, cstart_g, cfs, Rt, (T*)nullptr, done, cs, corr, stage, true);
+    return;
   }
-  if (stage >= 1 && !staged) mbar_wait_bounded(&bar, 0);  // no copy may land after the exit
+  pdl_wait();
+  if (done != nullptr && *done) return;
+  const int b = a - 1, per = (int)(blockDim.x >> 5);
+  scatter_items<T, TV>(((int)blockIdx.x - 1) * per + (int)(threadIdx.x >> 5), ((int)gridDim.x - 1) * per,
+                       N, P, ldN, nnz, b, a + 1, P - 1, rowptr, col, stack_km, kptr, klist, eptr, ek,
+                       eg, Rt + (size_t)b * ldN, 1, Rt);
 }
 
 // All eight phases of one column on a thread-block cluster of CL CTAs (grid = columns x CL): the
@@ -505,6 +543,47 @@ int launch_color_ilu(System& s, cudaStream_t st) {
   return check_launch("color_slots");
 }
 
+bool color_one_cta(const System& s) { return (s.N + 3) / 4 <= 2048; }
+
+// Shared memory of the one-CTA solve: the column, then the factors (1) and the coupling stencil
+// (2) where they fit.
+template <typename T>
+static int color_stage(const System& s, bool coupled, size_t& smem) {
+  smem = sizeof(T) * (size_t)s.ldN;
+  const size_t slots = kColorSlotBuf(s.N, sizeof(T));
+  if (smem + slots > kColorSmemMax) return 0;
+  smem += slots;
+  if (!coupled || smem + slots > kColorSmemMax) return 1;
+  smem += slots;
+  return 2;
+}
+
+template <typename T, typename TV>
+int launch_color_gs(System& s, int a, const T* lu, T* Rt, cudaStream_t st, const int* done,
+                    const T* cs, T* corr, const TV* stack_km, const T* eg) {
+  if (cs == nullptr || corr == nullptr || stack_km == nullptr)
+    return fail(SG_ERR_ARG, "four-colour sweep: no coupling tables");
+  size_t smem = 0;
+  const int stage = color_stage<T>(s, true, smem);
+  auto kern = color_gs_kernel<T, TV>;
+  SG_TRY(ensure_smem((const void*)kern, smem));
+  // a warp per (32-row tile, column) of block a - 1's scatter, on the SMs that the solve leaves
+  const long long items = a >= 1 ? (long long)((s.N + 31) / 32) * (s.P - 1 - a) : 0;
+  const int grid = 1 + (int)std::min(151LL, (items + 31) / 32);
+  TimeScope ts(s.timer, K_ILU_SOLVE, st);
+  return launch_pdl(kern, dim3(grid), dim3(1024), smem, st, s.pat.m, s.N, s.ldN, s.P, s.pat.nnz, a,
+                    s.cstart.p, lu, Rt, done, cs, corr, stage, s.rowptr.p, s.col.p, stack_km,
+                    s.gs_kptr.p, s.gs_k.p, s.gs_eptr.p, s.gs_ea.p, eg);
+}
+template int launch_color_gs<double, double>(System&, int, const double*, double*, cudaStream_t,
+                                             const int*, const double*, double*, const double*,
+                                             const double*);
+template int launch_color_gs<float, float>(System&, int, const float*, float*, cudaStream_t, const int*,
+                                           const float*, float*, const float*, const float*);
+template int launch_color_gs<float, __nv_bfloat16>(System&, int, const float*, float*, cudaStream_t,
+                                                   const int*, const float*, float*,
+                                                   const __nv_bfloat16*, const float*);
+
 // Block solves of columns a0 .. a0 + ncols - 1 from Rt into Z (colour-ordered factors).
 template <typename T>
 int launch_color_solve(System& s, int a0, int ncols, int fac_per_col, const T* lu, T* Rt, T* Z,
@@ -516,7 +595,7 @@ int launch_color_solve(System& s, int a0, int ncols, int fac_per_col, const T* l
   // one CTA with the column in shared memory below that.  A single-column solve with more than
   // 16384 nodes per colour takes a cluster of 16 where the device schedules one.
   const int per_colour = (s.N + 3) / 4;
-  if (per_colour > 2048) {
+  if (!color_one_cta(s)) {
     if (per_colour > 8 * 2048 && ncols == 1 && cluster16_ok<T>())
       return launch_cluster<T, 16>(s, a0, ncols, fac_per_col, lu, Rt, Z, st, done, cs, corr);
     if (per_colour > 4 * 2048)
@@ -525,37 +604,24 @@ int launch_color_solve(System& s, int a0, int ncols, int fac_per_col, const T* l
       return launch_cluster<T, 4>(s, a0, ncols, fac_per_col, lu, Rt, Z, st, done, cs, corr);
     return launch_cluster<T, 2>(s, a0, ncols, fac_per_col, lu, Rt, Z, st, done, cs, corr);
   }
-  {
-    // shared memory: the column, then the factors and the coupling stencil where they fit
-    int stage = 0;
-    size_t smem = sizeof(T) * (size_t)s.ldN;
-    const size_t slots = kColorSlotBuf(s.N, sizeof(T));
-    if (smem + slots <= kColorSmemMax) {
-      stage = 1;
-      smem += slots;
-      if (cs != nullptr && smem + slots <= kColorSmemMax) {
-        stage = 2;
-        smem += slots;
-      }
-    }
-    auto kern = color_cta_kernel<T>;
-    SG_TRY(ensure_smem((const void*)kern, smem));
-    TimeScope ts(s.timer, K_ILU_SOLVE, st);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)ncols, 1, 1);
-    cfg.blockDim = dim3(1024, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributePriority;
-    attr[0].val.priority = s.prio_hi;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    SG_CUDA(cudaLaunchKernelEx(&cfg, kern, m, s.N, s.ldN, s.P, a0, fac_per_col,
-                               (const int*)s.cstart.p, lu, Rt, Z, done, cs, corr, stage));
-    return check_launch("color_cta");
-  }
-  return fail(SG_ERR_ARG, "four-colour block solve: column larger than shared memory");
+  size_t smem = 0;
+  const int stage = color_stage<T>(s, cs != nullptr, smem);
+  auto kern = color_cta_kernel<T>;
+  SG_TRY(ensure_smem((const void*)kern, smem));
+  TimeScope ts(s.timer, K_ILU_SOLVE, st);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)ncols, 1, 1);
+  cfg.blockDim = dim3(1024, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributePriority;
+  attr[0].val.priority = s.prio_hi;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  SG_CUDA(cudaLaunchKernelEx(&cfg, kern, m, s.N, s.ldN, s.P, a0, fac_per_col,
+                             (const int*)s.cstart.p, lu, Rt, Z, done, cs, corr, stage));
+  return check_launch("color_cta");
 }
 
 template int launch_color_solve<double>(System&, int, int, int, const double*, double*, double*,

@@ -649,35 +649,9 @@ __global__ void __launch_bounds__(256) fs_scatter_direct_kernel(
     const T* __restrict__ eg, const T* __restrict__ zc, int zs, T* __restrict__ Rt,
     const int* __restrict__ done) {
   if (done != nullptr && *done) return;
-  const int lane = threadIdx.x & 31;
-  const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-  const int ntiles = (N + 31) / 32, na = a_hi - a_lo + 1;
-  const int k0 = kptr[b];
-  const int* ep = eptr + (size_t)b * (P + 1);
-  for (int item = gw; item < ntiles * na; item += nw) {
-    const int tile = item / na, a = a_lo + item % na;
-    const int q0 = ep[a], q1 = ep[a + 1];
-    if (q0 == q1) continue;
-    const int i = tile * 32 + lane;
-    const bool live = i < N;
-    const T r = live ? Rt[(size_t)a * ldN + i] : T(0);
-    const int e0 = live ? rowptr[i] : 0;
-    const int ne = live ? rowptr[i + 1] - e0 : 0;
-    T z[9];
-#pragma unroll
-    for (int e = 0; e < 9; ++e) z[e] = e < ne ? zc[(size_t)col[e0 + e] * zs] : T(0);
-    T s = T(0);
-    for (int q = q0; q < q1; ++q) {
-      const TV* ak = stack_km + (size_t)klist[k0 + ek[q]] * nnz + e0;
-      T t = T(0);
-#pragma unroll
-      for (int e = 0; e < 9; ++e)
-        if (e < ne) t += (T)ak[e] * z[e];
-      s += eg[q] * t;
-    }
-    if (live) Rt[(size_t)a * ldN + i] = r - s;
-  }
+  scatter_items<T, TV>((int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5),
+                       (int)((gridDim.x * blockDim.x) >> 5), N, P, ldN, nnz, b, a_lo, a_hi, rowptr,
+                       col, stack_km, kptr, klist, eptr, ek, eg, zc, zs, Rt);
 }
 
 // After block b, for the next column only: Rt[b+1, i] -= sum_k G_k[b+1,b] (A_k z_b)[i], one
@@ -873,6 +847,24 @@ int launch_scatter<float>(System& s, int b, bool next, const float* Z, float* Rt
                                         s.gs_eg_f32.p, Z, Rt, st, done);
 }
 
+// Block a of the sweep and the later-column scatter of block a - 1 in one launch (four-colour order,
+// a column per CTA).
+template <typename T>
+int launch_gs_step(System& s, int a, T* Rt, cudaStream_t st, const int* done);
+template <>
+int launch_gs_step<double>(System& s, int a, double* Rt, cudaStream_t st, const int* done) {
+  return launch_color_gs<double, double>(s, a, s.lu9.p, Rt, st, done, s.gsn_cs.p, s.gsn_corr.p,
+                                         s.stack_km.p, s.gs_eg.p);
+}
+template <>
+int launch_gs_step<float>(System& s, int a, float* Rt, cudaStream_t st, const int* done) {
+  if (s.prm.precision == SG_MIXED_BF16 || s.prm.coupling_bf16)
+    return launch_color_gs<float, __nv_bfloat16>(s, a, s.lu9_f32.p, Rt, st, done, s.gsn_cs32.p,
+                                                 s.gsn_corr32.p, s.stack_km16.p, s.gs_eg_f32.p);
+  return launch_color_gs<float, float>(s, a, s.lu9_f32.p, Rt, st, done, s.gsn_cs32.p,
+                                       s.gsn_corr32.p, s.stack_km32.p, s.gs_eg_f32.p);
+}
+
 // Field-split Gauss-Seidel: block a solved from column a of Rt, then its coupling subtracted from
 // the later columns.  Only column a + 1 must be complete before block a + 1 starts; with ``fork``
 // the scatter into columns a + 2 .. runs on the system's second stream, overlapping the solve of
@@ -882,13 +874,19 @@ int launch_scatter<float>(System& s, int b, bool next, const float* Z, float* Rt
 // the block solves (its stencil K_{a+1,a} assembled at setup): the solve of block a leaves
 // K_{a+1,a} z_a in a buffer that the solve of block a + 1 subtracts, and the solve of block a + 1
 // waits for the later-column scatter of block a - 1 instead; the solves leave z_a in column a of
-// Rt, and one transpose at the end writes D.
+// Rt, and one transpose at the end writes D.  Where one CTA solves a column, no second stream is
+// needed: block a and the later-column scatter of block a - 1 both need block a - 1 alone and share
+// a launch.
 template <typename T>
 int fs_gs_sweep(System& s, const T* R, T* D, T* Rt, cudaStream_t st, const int* done, bool fork) {
   SG_TRY(launch_columns<T>(s, R, Rt, st, done));
   cudaStream_t s2 = fork ? s.stream2 : st;
   const T* cs = PcBufs<T>::cs(s);
   if (s.prm.ilu_order == SG_ILU_COLOR4 && cs != nullptr) {
+    if (color_one_cta(s)) {
+      for (int a = 0; a < s.P; ++a) SG_TRY(launch_gs_step<T>(s, a, Rt, st, done));
+      return launch_rows<T>(s, Rt, D, st, done);
+    }
     for (int a = 0; a < s.P; ++a) {
       if (fork && a >= 2) SG_CUDA(cudaStreamWaitEvent(st, s.ev_r[(a - 2) & 1], 0));
       SG_TRY(launch_color_solve<T>(s, a, 1, 1, PcBufs<T>::lu9(s), Rt, (T*)nullptr, st, done, cs,

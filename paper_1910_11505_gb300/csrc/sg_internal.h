@@ -177,6 +177,44 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned by
       "l"(src), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
 }
+
+// Gauss-Seidel coupling of block b into the columns a_lo .. a_hi, one warp per (32-row tile, target
+// column): the items gw, gw + nw, ... of this warp.  The tables are those of fs_scatter_kernel.
+template <typename T, typename TV>
+__device__ __forceinline__ void scatter_items(
+    int gw, int nw, int N, int P, int ldN, int nnz, int b, int a_lo, int a_hi,
+    const int* __restrict__ rowptr, const int* __restrict__ col, const TV* __restrict__ stack_km,
+    const int* __restrict__ kptr, const int* __restrict__ klist, const int* __restrict__ eptr,
+    const int* __restrict__ ek, const T* __restrict__ eg, const T* __restrict__ zc, int zs,
+    T* __restrict__ Rt) {
+  const int lane = threadIdx.x & 31;
+  const int ntiles = (N + 31) / 32, na = a_hi - a_lo + 1;
+  const int k0 = kptr[b];
+  const int* ep = eptr + (size_t)b * (P + 1);
+  for (int item = gw; item < ntiles * na; item += nw) {
+    const int tile = item / na, a = a_lo + item % na;
+    const int q0 = ep[a], q1 = ep[a + 1];
+    if (q0 == q1) continue;
+    const int i = tile * 32 + lane;
+    const bool live = i < N;
+    const T r = live ? Rt[(size_t)a * ldN + i] : T(0);
+    const int e0 = live ? rowptr[i] : 0;
+    const int ne = live ? rowptr[i + 1] - e0 : 0;
+    T z[9];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) z[e] = e < ne ? zc[(size_t)col[e0 + e] * zs] : T(0);
+    T s = T(0);
+    for (int q = q0; q < q1; ++q) {
+      const TV* ak = stack_km + (size_t)klist[k0 + ek[q]] * nnz + e0;
+      T t = T(0);
+#pragma unroll
+      for (int e = 0; e < 9; ++e)
+        if (e < ne) t += (T)ak[e] * z[e];
+      s += eg[q] * t;
+    }
+    if (live) Rt[(size_t)a * ldN + i] = r - s;
+  }
+}
 #endif
 
 // ------------------------------------------------------------------ device buffers
@@ -467,6 +505,12 @@ int launch_color_solve(System& s, int a0, int ncols, int fac_per_col, const T* l
 // The next-column coupling stencils gsn_cs (FP64 systems) or gsn_cs32 (mixed systems, from the
 // BF16-rounded stiffness values when the sweep couples in BF16), from the FP64 k-major stack.
 int launch_color_coupling(System& s, cudaStream_t st);
+// Whether one CTA solves a column in the four-colour order, and then one step of the Gauss-Seidel
+// sweep: block a's solve beside the later-column scatter of block a - 1.
+bool color_one_cta(const System& s);
+template <typename T, typename TV>
+int launch_color_gs(System& s, int a, const T* lu, T* Rt, cudaStream_t st, const int* done,
+                    const T* cs, T* corr, const TV* stack_km, const T* eg);
 int launch_lu9(System& s, cudaStream_t st);
 // Natural-order solves of all columns by warps in FP32 (k_ilu_wave.cu): setup (wave_v stays empty
 // where they do not apply) and one application.
