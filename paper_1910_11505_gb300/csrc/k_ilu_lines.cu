@@ -122,7 +122,6 @@ __global__ void __launch_bounds__(kLineWarps * 64, 1) ilu_lines_kernel(
     int m, int N, int ldN, int P, int a0, int fac_per_col, const int* __restrict__ lev_off,
     const double* __restrict__ lu9, const double2* __restrict__ fac, const double* __restrict__ dinv,
     const double* __restrict__ Rt, double* Z, const int* __restrict__ done) {
-  if (done != nullptr && *done) return;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ LineBars bars;
   __shared__ int s_fail;
@@ -158,6 +157,10 @@ __global__ void __launch_bounds__(kLineWarps * 64, 1) ilu_lines_kernel(
       unsigned u = 0;
       for (; u < total; ++u) {
         const unsigned slot = u % kLineSlots;
+        if (u == kLineSlots) {  // the first slots are filled while the kernel before still runs
+          pdl_wait();
+          if (done != nullptr && *done) break;
+        }
         if (u >= kLineSlots &&
             (*vfail || !mbar_wait_bounded(&bars.empty[w][slot], ((u / kLineSlots) - 1u) & 1u))) {
           *vfail = 1;
@@ -171,6 +174,8 @@ __global__ void __launch_bounds__(kLineWarps * 64, 1) ilu_lines_kernel(
         mbar_wait_bounded(&bars.full[w][c % kLineSlots], (c / kLineSlots) & 1u);
     }
     __syncwarp();
+    pdl_wait();
+    if (done != nullptr && *done) return;
     // the boundary rows: their scaling by 1/u_ii
     for (int k = w * 32 + lane; k < 4 * (m - 1); k += warps * 32) {
       const int side = k / (m - 1), s = k - side * (m - 1);
@@ -181,6 +186,8 @@ __global__ void __launch_bounds__(kLineWarps * 64, 1) ilu_lines_kernel(
           rhs[x + m * y] * lu9[((size_t)set * 9 + 4) * N + lev_off[lv] + (y - ylo)];
     }
   } else {
+    pdl_wait();
+    if (done != nullptr && *done) return;
     const int r0 = 16 * w, nr = min(16, nx - r0);
     // the warp's lines, 16 loads a lane in flight
     for (int x = lane; x < nx; x += 32) {
@@ -283,10 +290,9 @@ int launch_lines_solve(System& s, int a0, int ncols, int fac_per_col, const doub
   if (ncols == 1) smem = std::max(smem, smem_optin_max() - 1024);
   SG_TRY(ensure_smem((const void*)ilu_lines_kernel, smem));
   TimeScope ts(s.timer, K_ILU_SOLVE, st);
-  ilu_lines_kernel<<<ncols, line_warps(nx) * 64, smem, st>>>(
-      s.pat.m, s.N, s.ldN, s.P, a0, fac_per_col, s.lev9_off.p, s.lu9.p,
-      reinterpret_cast<const double2*>(s.line_fac.p), s.line_dinv.p, Rt, Z, done);
-  return check_launch("ilu_lines");
+  return launch_pdl(ilu_lines_kernel, dim3(ncols), dim3(line_warps(nx) * 64), smem, st, s.pat.m, s.N, s.ldN,
+                    s.P, a0, fac_per_col, s.lev9_off.p, s.lu9.p,
+                    reinterpret_cast<const double2*>(s.line_fac.p), s.line_dinv.p, Rt, Z, done);
 }
 
 }  // namespace sg

@@ -18,9 +18,8 @@
 // writes inside the sweep had taken half of the time.
 //
 // Bound: the dependent chain of a step (a shuffle and two multiply-adds) and its instructions.
-// FP64 keeps the barrier kernels: four or five multiply-adds of 65 cycles each on one
-// sub-partition would bound a step here.  One application by 84 columns on one GB300, barrier kernels
-// -> here: 128 x 128 150 -> 74 us, 256 x 256 571 -> 123 us.
+// (FP64 spreads a row's four multiply-adds of 65 cycles over two lanes, k_ilu_lines.cu.)  One application by 84 columns on one GB300, barrier kernels
+// -> here: 32 x 32 41.5 -> 21 us, 128 x 128 150 -> 60 us, 256 x 256 571 -> 121 us.
 #include <algorithm>
 
 #include "sg_internal.h"
@@ -30,8 +29,8 @@ namespace sg {
 namespace {
 
 constexpr int kWaveMaxWarps = 8;   // compute warps: lines up to 256
-// Fewer lines go to the barrier kernels: 7 lines take 16.7 us there and 20.9 us here (62 steps of
-// idle lanes and a third launch), 15 lines 25.0 and 20.9, 31 lines 41.4 and 23.1.
+// Fewer lines go to the barrier kernels: 7 lines take 16 us there and 20 us here (62 steps of
+// idle lanes and a third launch), 15 lines 25.0 and 20.8, 31 lines 41.4 and 21.1.
 constexpr int kWaveMinLines = 12;
 constexpr int kWaveBlock = 8;      // steps of a ring slot
 constexpr int kWaveSlots = 4;

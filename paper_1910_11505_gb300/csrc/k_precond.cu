@@ -517,6 +517,7 @@ __global__ void __launch_bounds__(kTriMaxThreads) ilu_window_kernel(
 template <typename T>
 __global__ void columns_kernel(const T* __restrict__ R, T* __restrict__ Rt, int N, int P, int ld,
                                const int* __restrict__ done) {
+  pdl_trigger();
   if (done != nullptr && *done) return;
   __shared__ T tile[32][33];
   const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
@@ -666,6 +667,7 @@ __global__ void __launch_bounds__(256) fs_next_kernel(
     const int* __restrict__ klist, const int* __restrict__ eptr, const int* __restrict__ ek,
     const T* __restrict__ eg, const T* __restrict__ zcol, int zs, T* __restrict__ Rt,
     const int* __restrict__ done) {
+  pdl_trigger();  // the next block's solve may take its SM and fetch factors
   if (done != nullptr && *done) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
