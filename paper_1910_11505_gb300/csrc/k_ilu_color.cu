@@ -463,41 +463,277 @@ __global__ void __launch_bounds__(1024) color_cluster_kernel(
 
 
 
+// ---------------------------------------------------------------- column in the cluster's shared memory
+
+__device__ __forceinline__ void store_rank(unsigned addr, unsigned rank, float v) {
+  asm volatile("{\n\t.reg .u32 t;\n\tmapa.shared::cluster.u32 t, %0, %1;\n\tst.shared::cluster.f32 [t], %2;\n\t}\n" ::"r"(addr),
+               "r"(rank), "f"(v)
+               : "memory");
+}
+__device__ __forceinline__ void store_rank(unsigned addr, unsigned rank, double v) {
+  asm volatile("{\n\t.reg .u32 t;\n\tmapa.shared::cluster.u32 t, %0, %1;\n\tst.shared::cluster.f64 [t], %2;\n\t}\n" ::"r"(addr),
+               "r"(rank), "d"(v)
+               : "memory");
+}
+
+__host__ __device__ constexpr int split_rows(int m, int cl) { return (m + cl - 1) / cl; }
+
+// One CTA's share of a column: the lines y0 .. y0 + rows - 1 at w + m, a line of the neighbour on
+// either side.
+struct SplitGeom {
+  int m, N, P, a, y0, rows, per, rank;
+  // positions of colour (cx, cy) in these lines: cnt of them from pos0 on; their first line and width
+  __device__ __forceinline__ void colour(int C, const int* cstart, int& pos0, int& cnt, int& y1,
+                                         int& nx) const {
+    const int cx = C & 1, cy = C >> 1;
+    nx = (m - cx + 1) >> 1;
+    y1 = y0 + ((y0 ^ cy) & 1);
+    const int r = rows > y1 - y0 ? (rows - (y1 - y0) + 1) >> 1 : 0;
+    pos0 = cstart[C] + ((y1 - cy) >> 1) * nx;
+    cnt = r * nx;
+  }
+};
+
+// Factors of position pos that a phase uses (slot 4: 1/u_ii, or the previous column's coupling).
+template <typename T, int C, bool UPPER>
+__device__ __forceinline__ void split_fetch(int pos, int N, const T* __restrict__ cf, const T* corr,
+                                            T (&f)[9]) {
+#pragma unroll
+  for (int sl = 0; sl < 9; ++sl) {
+    const int cj = nb_colour(C, sl % 3 - 1, sl / 3 - 1);
+    if (sl == 4)
+      f[sl] = UPPER ? cf[(size_t)4 * N + pos] : corr != nullptr ? corr[pos] : T(0);
+    else if (UPPER ? cj > C : cj < C)
+      f[sl] = cf[(size_t)sl * N + pos];
+  }
+}
+
+// A thread's first positions of a phase (one in FP64, for the registers) have their factors fetched
+// before the barrier that the phase waits for.
+template <typename T>
+__host__ __device__ constexpr int split_n() { return sizeof(T) == 8 ? 1 : 2; }
+
+template <typename T, int C, bool UPPER>
+__device__ __forceinline__ void split_ahead(const SplitGeom& g, const int* cstart,
+                                            const T* __restrict__ cf, const T* corr,
+                                            T (&f)[split_n<T>()][9]) {
+  int pos0, cnt, y1, nx;
+  g.colour(C, cstart, pos0, cnt, y1, nx);
+#pragma unroll
+  for (int k = 0; k < split_n<T>(); ++k) {
+    const int q = (int)threadIdx.x + k * 1024;
+    if (q < cnt) split_fetch<T, C, UPPER>(pos0 + q, g.N, cf, corr, f[k]);
+  }
+}
+
+// One phase: the values of the CTA's nodes of colour C, and of its outer lines also in the
+// neighbours' copies.  The same arithmetic as color_node_value.
+template <typename T, int C, bool UPPER>
+__device__ __forceinline__ void split_phase(const SplitGeom& g, const int* cstart,
+                                            const T* __restrict__ cf, const T* corr, T* w,
+                                            T (&f)[split_n<T>()][9]) {
+  int pos0, cnt, y1, nx;
+  g.colour(C, cstart, pos0, cnt, y1, nx);
+  const int m = g.m;
+  auto node = [&](int q, const T(&fq)[9]) {
+    int r = (int)((float)q * __frcp_rn((float)nx));
+    int rem = q - r * nx;
+    if (rem < 0) {
+      --r;
+      rem += nx;
+    } else if (rem >= nx) {
+      ++r;
+      rem -= nx;
+    }
+    const int y = y1 + 2 * r, x = (C & 1) + 2 * rem;
+    T* line = w + (y - g.y0 + 1) * m;
+    const int xl = max(x - 1, 0), xr = min(x + 1, m - 1);
+    const int yd = y > 0 ? -m : 0, yu = y < m - 1 ? m : 0;
+    T v = line[x];
+    if (UPPER) v *= fq[4];
+    else if (corr != nullptr) v -= fq[4];
+#pragma unroll
+    for (int sl = 0; sl < 9; ++sl) {
+      if (sl == 4) continue;
+      const int dx = sl % 3 - 1, dy = sl / 3 - 1;
+      const int cj = nb_colour(C, dx, dy);
+      if (UPPER ? cj <= C : cj >= C) continue;
+      v -= fq[sl] * line[(dx < 0 ? xl : dx > 0 ? xr : x) + (dy < 0 ? yd : dy > 0 ? yu : 0)];
+    }
+    line[x] = v;
+    if (y == g.y0 && y > 0) store_rank(smem_u32(w + (g.per + 1) * m + x), g.rank - 1, v);
+    if (y == g.y0 + g.rows - 1 && y < m - 1) store_rank(smem_u32(w + x), g.rank + 1, v);
+  };
+#pragma unroll
+  for (int k = 0; k < split_n<T>(); ++k) {
+    const int q = (int)threadIdx.x + k * 1024;
+    if (q < cnt) node(q, f[k]);
+  }
+  for (int q = (int)threadIdx.x + split_n<T>() * 1024; q < cnt; q += 1024) {
+    T fq[9];
+    split_fetch<T, C, UPPER>(pos0 + q, g.N, cf, corr, fq);
+    node(q, fq);
+  }
+}
+
+template <typename T, int C>
+__device__ __forceinline__ void split_coupling(const SplitGeom& g, const int* cstart,
+                                               const T* __restrict__ csn, const T* w, T* corr) {
+  int pos0, cnt, y1, nx;
+  g.colour(C, cstart, pos0, cnt, y1, nx);
+  const int m = g.m;
+  for (int q = threadIdx.x; q < cnt; q += 1024) {
+    const int r = q / nx, y = y1 + 2 * r, x = (C & 1) + 2 * (q - r * nx);
+    const T* line = w + (y - g.y0 + 1) * m;
+    const int xl = max(x - 1, 0), xr = min(x + 1, m - 1);
+    const int yd = y > 0 ? -m : 0, yu = y < m - 1 ? m : 0;
+    T s = T(0);
+#pragma unroll
+    for (int sl = 0; sl < 9; ++sl) {
+      const int dx = sl % 3 - 1, dy = sl / 3 - 1;
+      s += csn[(size_t)sl * g.N + pos0 + q] *
+           line[(dx < 0 ? xl : dx > 0 ? xr : x) + (dy < 0 ? yd : dy > 0 ? yu : 0)];
+    }
+    corr[pos0 + q] = s;
+  }
+}
+
+// The solve of color_cluster_kernel with the column in the cluster's shared memory: a CTA owns a range
+// of lines, works on them there, and stores its outer lines' new values into the neighbour CTA's copy as
+// well (nothing of a colour is read in the phase that writes it), so that every read is local
+// and a phase's barrier orders shared memory alone; the factors of the next phase are on their way
+// before the barrier.
+// Bound: the latency of eight phases and their barriers.  Measured on one GB300: the figures stand at
+// the rule in launch_color_solve.
+template <typename T, int CL>
+__global__ void __launch_bounds__(1024) color_split_kernel(
+    int m, int N, int ldN, int P, int a0, int fac_per_col, const int* __restrict__ cstart_g,
+    const T* __restrict__ cfs, T* __restrict__ Rt, T* __restrict__ Z, const int* __restrict__ done,
+    const T* __restrict__ cs, T* corr) {
+  if (done != nullptr && *done) return;  // uniform over the cluster: no barrier is skipped by some
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* w = reinterpret_cast<T*>(smem_raw);  // (per + 2) x m
+  __shared__ int cstart[5];
+  SplitGeom g;
+  g.m = m;
+  g.N = N;
+  g.P = P;
+  g.a = a0 + blockIdx.x / CL;
+  g.rank = blockIdx.x % CL;
+  g.per = split_rows(m, CL);
+  g.y0 = g.rank * g.per;
+  g.rows = max(0, min(m - g.y0, g.per));
+  const int a = g.a;
+  const T* cf = cfs + (size_t)(fac_per_col ? a : 0) * 9 * N;
+  T* rhs = Rt + (size_t)a * ldN + (size_t)g.y0 * m;
+  const T* corr_in = (cs != nullptr && a > 0) ? corr : nullptr;
+  const T* csn = (cs != nullptr && a + 1 < P) ? cs + (size_t)a * 9 * N : nullptr;
+  if (gridDim.x == CL) {
+    l2_prefetch(cf, sizeof(T) * 9 * (size_t)N, g.rank, CL);
+    if (csn != nullptr) l2_prefetch(csn, sizeof(T) * 9 * (size_t)N, g.rank, CL);
+  }
+  if (threadIdx.x < 5) cstart[threadIdx.x] = cstart_g[threadIdx.x];
+  const int n = g.rows * m;
+  for (int i = threadIdx.x; i < n; i += 1024) w[m + i] = rhs[i];
+  __syncthreads();
+  auto arrive = []() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); };
+  auto wait = []() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); };
+  T f[split_n<T>()][9];
+  arrive();
+  split_ahead<T, 0, false>(g, cstart, cf, corr_in, f);
+  wait();
+  split_phase<T, 0, false>(g, cstart, cf, corr_in, w, f);
+  arrive();
+  split_ahead<T, 1, false>(g, cstart, cf, corr_in, f);
+  wait();
+  split_phase<T, 1, false>(g, cstart, cf, corr_in, w, f);
+  arrive();
+  split_ahead<T, 2, false>(g, cstart, cf, corr_in, f);
+  wait();
+  split_phase<T, 2, false>(g, cstart, cf, corr_in, w, f);
+  arrive();
+  split_ahead<T, 3, false>(g, cstart, cf, corr_in, f);
+  wait();
+  split_phase<T, 3, false>(g, cstart, cf, corr_in, w, f);
+  arrive();
+  split_ahead<T, 3, true>(g, cstart, cf, (const T*)nullptr, f);
+  wait();
+  split_phase<T, 3, true>(g, cstart, cf, (const T*)nullptr, w, f);
+  arrive();
+  split_ahead<T, 2, true>(g, cstart, cf, (const T*)nullptr, f);
+  wait();
+  split_phase<T, 2, true>(g, cstart, cf, (const T*)nullptr, w, f);
+  arrive();
+  split_ahead<T, 1, true>(g, cstart, cf, (const T*)nullptr, f);
+  wait();
+  split_phase<T, 1, true>(g, cstart, cf, (const T*)nullptr, w, f);
+  arrive();
+  split_ahead<T, 0, true>(g, cstart, cf, (const T*)nullptr, f);
+  wait();
+  split_phase<T, 0, true>(g, cstart, cf, (const T*)nullptr, w, f);
+  arrive();
+  wait();  // no CTA stores into another's memory from here on
+  for (int i = threadIdx.x; i < n; i += 1024) {
+    rhs[i] = w[m + i];
+    if (Z != nullptr) Z[((size_t)g.y0 * m + i) * P + a] = w[m + i];
+  }
+  if (csn != nullptr) {
+    split_coupling<T, 0>(g, cstart, csn, w, corr);
+    split_coupling<T, 1>(g, cstart, csn, w, corr);
+    split_coupling<T, 2>(g, cstart, csn, w, corr);
+    split_coupling<T, 3>(g, cstart, csn, w, corr);
+  }
+}
+
+template <typename T>
+using ClusterKern = void (*)(int, int, int, int, int, int, const int*, const T*, T*, T*, const int*,
+                             const T*, T*);
+
 // Whether clusters of 16 CTAs of 1024 threads (a non-portable size) can be scheduled on this
 // device: asked once per process and kernel; on any failure the answer is no.
 template <typename T>
-bool cluster16_ok() {
-  static int ok = -1;
-  if (ok < 0) {
-    ok = 0;
-    auto kern = color_cluster_kernel<T, 16>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(16, 1, 1);
-      cfg.blockDim = dim3(1024, 1, 1);
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = 16;
-      attr[0].val.clusterDim.y = 1;
-      attr[0].val.clusterDim.z = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      int nclusters = 0;
-      if (cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg) == cudaSuccess && nclusters >= 2)
-        ok = 1;
-    }
-    cudaGetLastError();
+bool cluster16_ok(ClusterKern<T> kern, size_t smem) {
+  bool ok = false;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+      ensure_smem((const void*)kern, smem) == SG_OK) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(16, 1, 1);
+    cfg.blockDim = dim3(1024, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 16;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int nclusters = 0;
+    ok = cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg) == cudaSuccess && nclusters >= 2;
   }
-  return ok == 1;
+  cudaGetLastError();
+  return ok;
+}
+
+// Shared memory of color_split_kernel; 0 where a CTA's lines do not fit (color_cluster_kernel then).
+template <typename T>
+size_t split_smem(int m, int cl) {
+  const size_t b = sizeof(T) * (size_t)(split_rows(m, cl) + 2) * m;
+  return b <= kColorSmemMax ? b : 0;
 }
 
 template <typename T, int CL>
 int launch_cluster(System& s, int a0, int ncols, int fac_per_col, const T* lu, T* Rt, T* Z,
-                   cudaStream_t st, const int* done, const T* cs, T* corr) {
+                   cudaStream_t st, const int* done, const T* cs, T* corr, bool split) {
+  const size_t smem = split ? split_smem<T>(s.pat.m, CL) : 0;
+  ClusterKern<T> kern = color_cluster_kernel<T, CL>;
+  if (smem > 0) {
+    kern = color_split_kernel<T, CL>;
+    SG_TRY(ensure_smem((const void*)kern, smem));
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(ncols * CL), 1, 1);
   cfg.blockDim = dim3(1024, 1, 1);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -509,8 +745,8 @@ int launch_cluster(System& s, int a0, int ncols, int fac_per_col, const T* lu, T
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   TimeScope ts(s.timer, K_ILU_SOLVE, st);
-  SG_CUDA(cudaLaunchKernelEx(&cfg, color_cluster_kernel<T, CL>, s.pat.m, s.N, s.ldN, s.P, a0,
-                             fac_per_col, (const int*)s.cstart.p, lu, Rt, Z, done, cs, corr));
+  SG_CUDA(cudaLaunchKernelEx(&cfg, kern, s.pat.m, s.N, s.ldN, s.P, a0, fac_per_col,
+                             (const int*)s.cstart.p, lu, Rt, Z, done, cs, corr));
   return check_launch("color_cluster");
 }
 
@@ -584,6 +820,14 @@ template int launch_color_gs<float, __nv_bfloat16>(System&, int, const float*, f
                                                    const int*, const float*, float*,
                                                    const __nv_bfloat16*, const float*);
 
+// The largest split form whose 16 CTAs are asked for is the largest that fits.
+template <typename T>
+static bool clusters16(int m, bool in_smem) {
+  static const bool split = cluster16_ok<T>(color_split_kernel<T, 16>, kColorSmemMax);
+  static const bool plain = cluster16_ok<T>(color_cluster_kernel<T, 16>, 0);
+  return in_smem && split_smem<T>(m, 16) > 0 ? split : plain;
+}
+
 // Block solves of columns a0 .. a0 + ncols - 1 from Rt into Z (colour-ordered factors).
 template <typename T>
 int launch_color_solve(System& s, int a0, int ncols, int fac_per_col, const T* lu, T* Rt, T* Z,
@@ -591,18 +835,25 @@ int launch_color_solve(System& s, int a0, int ncols, int fac_per_col, const T* l
   if (cs != nullptr && (ncols != 1 || corr == nullptr))
     return fail(SG_ERR_ARG, "four-colour solve: the coupled form takes one column and a buffer");
   const int m = s.pat.m;
-  // a cluster of CTAs once one CTA would hold more than ~2048 nodes per colour (two per thread);
-  // one CTA with the column in shared memory below that.  A single-column solve with more than
-  // 16384 nodes per colour takes a cluster of 16 where the device schedules one.
-  const int per_colour = (s.N + 3) / 4;
+  // One CTA with the column in shared memory up to 2048 nodes per colour (two per thread), else a
+  // cluster of CTAs, 16 of them only where the device schedules them.  The column in the
+  // cluster's shared memory and one node per thread for a single column (20 Gauss-Seidel blocks
+  // FP32: 100 lines 594 us in L2, 504 split over half as many CTAs, 401; 200 lines 817, 729, 600; FP64
+  // 1093, 995, 709 and 1540, 1362, 1078); for all columns at once two nodes per thread (FP32 128
+  // lines: 27 us in L2, 23.5, 30.3).  FP64 stays in L2 for all columns (128 lines: 35.5 us, split
+  // 38) and beyond 16384 nodes per colour (256 lines, 20 blocks: 1601 us, split 1667), where its
+  // threads have several nodes, and registers for the factors of one.
   if (!color_one_cta(s)) {
-    if (per_colour > 8 * 2048 && ncols == 1 && cluster16_ok<T>())
-      return launch_cluster<T, 16>(s, a0, ncols, fac_per_col, lu, Rt, Z, st, done, cs, corr);
-    if (per_colour > 4 * 2048)
-      return launch_cluster<T, 8>(s, a0, ncols, fac_per_col, lu, Rt, Z, st, done, cs, corr);
-    if (per_colour > 2 * 2048)
-      return launch_cluster<T, 4>(s, a0, ncols, fac_per_col, lu, Rt, Z, st, done, cs, corr);
-    return launch_cluster<T, 2>(s, a0, ncols, fac_per_col, lu, Rt, Z, st, done, cs, corr);
+    const int per_colour = (s.N + 3) / 4;
+    const bool split = sizeof(T) == 4 || (ncols == 1 && per_colour <= 8 * 2048);
+    const int load = split && ncols == 1 ? 2 * per_colour : per_colour;
+    if (load > 8 * 2048 && ncols == 1 && clusters16<T>(m, split))
+      return launch_cluster<T, 16>(s, a0, ncols, fac_per_col, lu, Rt, Z, st, done, cs, corr, split);
+    if (load > 4 * 2048)
+      return launch_cluster<T, 8>(s, a0, ncols, fac_per_col, lu, Rt, Z, st, done, cs, corr, split);
+    if (load > 2 * 2048)
+      return launch_cluster<T, 4>(s, a0, ncols, fac_per_col, lu, Rt, Z, st, done, cs, corr, split);
+    return launch_cluster<T, 2>(s, a0, ncols, fac_per_col, lu, Rt, Z, st, done, cs, corr, split);
   }
   size_t smem = 0;
   const int stage = color_stage<T>(s, cs != nullptr, smem);
