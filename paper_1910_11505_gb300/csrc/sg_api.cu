@@ -1080,7 +1080,6 @@ int sg_setup(const sg_params* prm, int nsys, void* stream, sg_handle** out) {
     sg_handle* h = new sg_handle();
     cudaGetDevice(&h->device);
     int rc = SG_OK;
-    bool blocks = false;
     for (int i = 0; i < nsys && rc == SG_OK; ++i) {
       System* s = new System();
       s->prm = prm[i];
@@ -1088,8 +1087,6 @@ int sg_setup(const sg_params* prm, int nsys, void* stream, sg_handle** out) {
       s->lean = lean;
       h->sys.push_back(s);
       rc = setup_system(*s, st);
-      blocks = blocks || s->block64.ready || s->block32.ready || s->wave_low.p != nullptr ||
-               s->line_fac.p != nullptr;
       if (rc != SG_OK) fail(rc, "system " + std::to_string(i) + ": " + std::string(g_last_error));
     }
     if (rc == SG_OK) rc = make_pool(h, st);
@@ -1099,7 +1096,7 @@ int sg_setup(const sg_params* prm, int nsys, void* stream, sg_handle** out) {
     }
     const std::string msg = g_last_error;
     sg_free(h);
-    if (rc != SG_ERR_OOM || !blocks) return fail(rc, msg);
+    if (rc != SG_ERR_OOM || lean) return fail(rc, msg);
   }
   return fail(SG_ERR_OOM, "out of memory");
 }

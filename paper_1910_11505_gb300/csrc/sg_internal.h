@@ -375,7 +375,7 @@ struct System {
   DBuf<float> ent_g_f32;
   TileOp tile64, tile32;       // row-tiled operator in FP64 / FP32 (when built)
   BlockOp block64, block32;    // block-stencil operator in FP64 / FP32 (when built)
-  bool lean = false;           // set up again without the block-stencil operator (out of memory)
+  bool lean = false;           // set up again (out of memory): no block-stencil operator, no factor streams
   std::string tile_msg;        // why a row-tiled operator was not built (empty if it was)
   // device: preconditioner
   int nfac = 0;                // number of factor sets (1 for mean, P for field split)
