@@ -11,8 +11,8 @@
 // stride ldN, filled from the N x P residual by a tiled transpose).  The ILU(0) triangular solves
 // run as wavefronts: rows of one level of the lower (upper) graph of the pattern depend only on
 // rows of earlier levels; one CTA owns one chaos column and walks all levels with a CTA barrier
-// in between, keeping only a window of level rows in shared memory, so any mesh takes the same
-// path.  The off-diagonal coupling of the Gauss-Seidel sweep, sum_{b<a} K_ab z_b, is subtracted
+// in between, keeping the column or a window of level rows in shared memory, so any mesh can take
+// this path; most sizes have a faster one (FP32, all columns: k_ilu_wave.cu; FP64: k_ilu_lines.cu).  The off-diagonal coupling of the Gauss-Seidel sweep, sum_{b<a} K_ab z_b, is subtracted
 // from the later columns of rhs_t after each block b by a grid-wide kernel:
 // T[k] = sum_e A[e,k] z_b[j_e] once per (row, k), then rhs_t[a] -= G_k[a,b] T[k] for a > b.
 #include <algorithm>

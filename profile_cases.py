@@ -1,6 +1,6 @@
 """Small, self-contained cases of single kernels for profiling (e.g. under ``ncu``).
 
-    python profile_cases.py precond [fs_gs|fs_jacobi|mean] [n]
+    python profile_cases.py precond [fs_gs|fs_jacobi|mean] [n] [fp64|fp32]
     python profile_cases.py sweep [n] [M] [p] [fp32|fp64]   # four-colour FS-GS sweep as in c3
     python profile_cases.py vcycle [reps] [fg|fs_gs]   # the c3 mixed solve's V-cycle preconditioner
     python profile_cases.py smoother [fg|fs_gs] [n]     # the c3 smoother alone on an n x n mesh
@@ -61,12 +61,17 @@ def main(argv):
     if what == "precond":
         pc = argv[2] if len(argv) > 2 else "fs_gs"
         n = int(argv[3]) if len(argv) > 3 else 128
-        h = sg.sg_setup(sg.sg_default_params(n=n, M=4, p=3, sigma=0.5, ell=0.5, precond=pc))
+        prec = argv[4] if len(argv) > 4 else "fp64"
+        h = sg.sg_setup(sg.sg_default_params(n=n, M=4, p=3, sigma=0.5, ell=0.5, precond=pc,
+                                             precision=prec))
         N, P, _ = sg.sg_dims(h)
         R = torch.from_numpy(W.random_field(N, P, seed=1)).cuda()
+        if prec == "fp32":
+            R = R.float()
         Z = torch.empty_like(R)
+        apply = sg.sg_precond_apply_lowp if prec == "fp32" else sg.sg_precond_apply
         for _ in range(3):
-            sg.sg_precond_apply(h, 0, R, Z)
+            apply(h, 0, R, Z)
     elif what == "sweep":
         # the field-split Gauss-Seidel sweep of the c3 smoother (four-colour ILU(0); the FP32
         # form couples from the BF16 stiffness copy)
