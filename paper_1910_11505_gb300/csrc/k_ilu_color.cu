@@ -695,7 +695,7 @@ template <typename T>
 bool cluster16_ok(ClusterKern<T> kern, size_t smem) {
   bool ok = false;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-      ensure_smem((const void*)kern, smem) == SG_OK) {
+      (smem == 0 || ensure_smem((const void*)kern, smem) == SG_OK)) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(16, 1, 1);
     cfg.blockDim = dim3(1024, 1, 1);
