@@ -300,27 +300,26 @@ __global__ void __launch_bounds__(544, 1) tc_train_kernel(
     const int j0 = (blockIdx.x + n * S) * kTcUnits;
     return j0 + kTcTRow <= out && (j0 >= 4 || (tw & 3u) == 0);
   };
-  // 16-byte chunks tid, tid + 512, ... of the block's rows x 33: place in T (of tile 0) or ~0
+  // 16-byte chunks tid, tid + 512, ... of the block's rows x 33: place in T (of tile 0), or null.
+  // (Pointers: a row of the block starts up to 127 x 4 out bytes in, past 4 GB from out = 8.5 M on.)
   constexpr int kChunks = kTcTRow / 4, kMine = (kTcRows * kChunks + 511) / 512;
-  const unsigned char* t_al = reinterpret_cast<const unsigned char*>(
-      reinterpret_cast<unsigned long long>(T + (size_t)b0 * out) & ~15ull);
-  unsigned toff[kMine];
+  const unsigned char* tsrc[kMine];
 #pragma unroll
   for (int k = 0; k < kMine; ++k) {
     const int c = (tid & 511) + 512 * k, r = c / kChunks;
     const unsigned long long row = reinterpret_cast<unsigned long long>(T + (size_t)(b0 + r) * out) & ~15ull;
-    toff[k] = r < kTcRows && b0 + r < B
-                  ? (unsigned)(row - reinterpret_cast<unsigned long long>(t_al)) + 16u * (c - r * kChunks)
-                  : ~0u;
+    tsrc[k] = r < kTcRows && b0 + r < B
+                  ? reinterpret_cast<const unsigned char*>(row) + 16 * (c - r * kChunks)
+                  : nullptr;
   }
   auto load_t = [&](int n) {
     if (n < n_tiles && bulk_t(n)) {
-      const unsigned char* src = t_al + (size_t)(blockIdx.x + n * S) * (kTcUnits * 4);
+      const size_t at = (size_t)(blockIdx.x + n * S) * (kTcUnits * 4);
       const unsigned dst = smem_u32(Tb) + (n & 1) * kTcTBytes + 16u * tid;
 #pragma unroll
       for (int k = 0; k < kMine; ++k)
-        if (toff[k] != ~0u)
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + 8192u * k), "l"(src + toff[k])
+        if (tsrc[k] != nullptr)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + 8192u * k), "l"(tsrc[k] + at)
                        : "memory");
     }
     // (arrives when this thread's copies so far have landed)
