@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(544, 1) tc_train_kernel(
                      *tfull = bar + 6;  // of 2, 1, 2, 1 and 2
   unsigned* tslot = reinterpret_cast<unsigned*>(bar + 8);
   volatile int* vfail = reinterpret_cast<volatile int*>(bar + 9);
-  float* red = reinterpret_cast<float*>(bar + 10);  // 16
+  double* red = reinterpret_cast<double*>(bar + 10);  // 16
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int b0 = blockIdx.y * kTcRows, S = gridDim.x;
   const int ntiles = (out + kTcUnits - 1) / kTcUnits;
@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(544, 1) tc_train_kernel(
   auto wait = [&](unsigned long long* b, int phase) {
     if (!*vfail && !mbar_wait_bounded(b, (unsigned)(phase & 1))) *vfail = 1;
   };
-  float lsum = 0.0f;
+  double lsum = 0.0;  // of the tiles' FP32 sums (a thread has 32 squares a tile, thousands in all)
   if (warp == 16) {
     if (lane == 0) {
       const unsigned ha = smem_u32(Ht), wa = smem_u32(Wt), da = smem_u32(Dy);
@@ -427,6 +427,7 @@ __global__ void __launch_bounds__(544, 1) tc_train_kernel(
       }
       const int sh1 = bulk ? shift[1] : shift[0], sh2 = bulk ? shift[2] : shift[0],
                 sh3 = bulk ? shift[3] : shift[0];
+      float tsum = 0.0f;
       // (units beyond the layer have W3 = b3 = T = 0, rows beyond the batch are masked)
 #pragma unroll
       for (int hf = 0; hf < 32; hf += 16) {
@@ -439,11 +440,12 @@ __global__ void __launch_bounds__(544, 1) tc_train_kernel(
           float r1 = (__uint_as_float(v[q + 1]) + bias) - t2[kTcTRow + (q & 2 ? sh3 : sh1)];
           if (hf + q >= nrow) r0 = 0.0f;
           if (hf + q + 1 >= nrow) r1 = 0.0f;
-          lsum = fmaf(r0, r0, lsum);
-          lsum = fmaf(r1, r1, lsum);
+          tsum = fmaf(r0, r0, tsum);
+          tsum = fmaf(r1, r1, tsum);
           dy[(hf + q) / 2] = __floats2bfloat162_rn(scale * r0, scale * r1);
         }
       }
+      lsum += (double)tsum;
       bias = bias_next;
       asm volatile("bar.sync 1, 512;\n" ::: "memory");  // every warp has read this T buffer
       load_t(n + 2);
@@ -490,9 +492,9 @@ __global__ void __launch_bounds__(544, 1) tc_train_kernel(
                  : "memory");
   }
   if (tid == 0) {
-    float l = 0.0f;
+    double l = 0.0;
     for (int i = 0; i < 16; ++i) l += red[i];
-    lpart[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = l;
+    lpart[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = (float)l;
   }
 }
 
