@@ -28,8 +28,10 @@
 // 4.25 ms (2.3 G multiply-adds, 1.09 TFLOP/s) against 19.3 ms; n = 128, P = 35 FP64 0.206 ms
 // against 0.917 ms.  The tiles take 2.2 times the row-tiled stack's memory at P = 84, L = 924.
 //
-// Every wait is bounded: after kWaitLimit polls the CTA raises the error word, stops waiting,
-// lets its copies in flight land (bounded) and writes NaN.
+// Every wait is bounded: after wait_limit polls (kWaitLimit, unless a test asks for fewer) the CTA
+// raises the error word, stops waiting, lets its copies in flight land (bounded by kWaitLimit) and
+// writes NaN.  A warp that has given up no longer arrives on the empty barriers: it would run ahead
+// of the others, and two arrivals of a diagonal tile on a barrier that waits for one are undefined.
 #include <algorithm>
 
 #include "sg_internal.h"
@@ -47,6 +49,7 @@ struct BlockArgs {
   int N, m, P, nb, rounds, ntile, ntiles_row, slots;
   long long item_elems;
   int evict_first;
+  long long wait_limit;  // polls after which a wait between the CTA's warps gives up
 };
 
 template <typename T>
@@ -128,6 +131,12 @@ __global__ void __launch_bounds__((kBlockMaxWarps + 1) * 32) block_edge_kernel(
     if (lane == 0) {
       unsigned cnt = 0;
       bool ok = true;
+      auto wait_room = [&](unsigned long long* bar, unsigned parity) {
+        if (mbar_try_wait(bar, parity)) return true;
+        for (long long n = 0; n < g.wait_limit && !*vfail; ++n)
+          if (mbar_try_wait(bar, parity)) return true;
+        return false;
+      };
       for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
         const T* src = K + (size_t)it * g.item_elems;
         for (int s = 0; s < g.ntile; ++s, ++cnt) {
@@ -140,7 +149,7 @@ __global__ void __launch_bounds__((kBlockMaxWarps + 1) * 32) block_edge_kernel(
           }
           const int slot = (int)(cnt & slot_mask);
           if (cnt >= (unsigned)g.slots &&
-              !mbar_wait_bounded(&empty[slot], ((cnt >> slot_log) - 1u) & 1u)) {
+              !wait_room(&empty[slot], ((cnt >> slot_log) - 1u) & 1u)) {
             *vfail = 1;
             ok = false;
             break;
@@ -186,11 +195,10 @@ __global__ void __launch_bounds__((kBlockMaxWarps + 1) * 32) block_edge_kernel(
   auto wait_tile = [&](unsigned c, int slot) {
     for (long long n = 0; (int)(issued - c) <= 0; ++n) {
       issued = *vissued;
-      if (n >= kWaitLimit) return false;
-      if (*vfail) return false;
+      if (n >= g.wait_limit || *vfail) return false;
     }
     __threadfence_block();
-    return mbar_wait_bounded(&full[slot], (c >> slot_log) & 1u);
+    return mbar_wait_bounded(&full[slot], (c >> slot_log) & 1u, g.wait_limit);
   };
   if (sizeof(T) == 4 && (int)blockIdx.x < nitems) fetch(blockIdx.x);
   for (int it = blockIdx.x; it < nitems; it += gridDim.x, base += (unsigned)g.ntile) {
@@ -218,7 +226,8 @@ __global__ void __launch_bounds__((kBlockMaxWarps + 1) * 32) block_edge_kernel(
       const int en = tab[r * nb + w];
       const unsigned c = base + (unsigned)(en & 0xffff);
       const int slot = (int)(c & slot_mask), kind = en >> 24;
-      if (!*vfail && !wait_tile(c, slot)) *vfail = 1;
+      const bool got = !*vfail && wait_tile(c, slot);
+      if (!got) *vfail = 1;
       const T* k = ring + (size_t)slot * kPair * kBR + lane;
       const T* db = D + (size_t)((en >> 16) & 0xff) * TS * kBLd + lane;
       T d[TS];
@@ -245,7 +254,7 @@ __global__ void __launch_bounds__((kBlockMaxWarps + 1) * 32) block_edge_kernel(
           }
       }
       __syncwarp();
-      if (lane == 0) mbar_arrive_n(&empty[slot], kind == 2 ? 2u : 1u);
+      if (lane == 0 && got) mbar_arrive_n(&empty[slot], kind == 2 ? 2u : 1u);
     }
     bar();  // every warp has read the differences: f takes their place
     if (*vfail) {
@@ -571,7 +580,8 @@ int launch_block_op(const System& s, const BlockOp& op, const T* X, T* Y, T alph
                     T beta, T* F, cudaStream_t st, const int* done) {
   if (!op.ready || F == nullptr) return fail(SG_ERR_ARG, "block operator not built");
   const BlockArgs g{s.N, s.pat.m, s.P, op.nb, op.rounds, op.ntile, op.row_tiles, op.slots,
-                    (long long)op.nval * kBR, op.bytes > ((size_t)64 << 20) ? 1 : 0};
+                    (long long)op.nval * kBR, op.bytes > ((size_t)64 << 20) ? 1 : 0,
+                    test_wait_limit()};
   auto kern = block_kernel<T>(op.TS);
   TimeScope ts(s.timer, sizeof(T) == 8 ? K_APPLY_F64 : K_APPLY_LOWP, st);
   SG_TRY(launch_pdl(kern, dim3(op.grid), dim3((op.nb + 1) * 32), op.smem, st, g, (const int*)op.table.p,

@@ -61,6 +61,10 @@ size_t smem_optin_max() {
   return (size_t)v;
 }
 
+// What the tests of failure paths set on their own thread (sg_test_hook).
+static thread_local long long g_test_wait = -1;
+long long test_wait_limit() { return g_test_wait >= 0 ? g_test_wait : kWaitLimit; }
+
 TimeScope::TimeScope(Timer* t_, int cls_, cudaStream_t st_) : t(t_), cls(cls_), st(st_) {
   if (!t || !t->on) return;
   long long c = t->count[cls]++;
@@ -1336,6 +1340,14 @@ void sg_free(sg_handle* h) {
   for (auto& e : h->timer.ev) cudaEventDestroy(e);
   if (h->pool) cudaMemPoolDestroy(h->pool);
   delete h;
+}
+
+// For the tests of failure paths; acts on the calling thread alone.  what 0: polls after which the
+// block-stencil operator's waits give up (0: at once; negative: the usual limit).
+int sg_test_hook(int what, long long value) {
+  if (what != 0) return fail(SG_ERR_ARG, "unknown hook");
+  g_test_wait = value;
+  return SG_OK;
 }
 
 const char* sg_last_error(void) { return g_last_error.c_str(); }
