@@ -28,10 +28,10 @@
 // 4.25 ms (2.3 G multiply-adds, 1.09 TFLOP/s) against 19.3 ms; n = 128, P = 35 FP64 0.206 ms
 // against 0.917 ms.  The tiles take 2.2 times the row-tiled stack's memory at P = 84, L = 924.
 //
-// Every wait is bounded: after wait_limit polls (kWaitLimit, unless a test asks for fewer) the CTA
-// raises the error word, stops waiting, lets its copies in flight land (bounded by kWaitLimit) and
-// writes NaN.  A warp that has given up no longer arrives on the empty barriers: it would run ahead
-// of the others, and two arrivals of a diagonal tile on a barrier that waits for one are undefined.
+// Every wait is bounded: after kWaitLimit polls the CTA raises the error word, stops waiting,
+// lets its copies in flight land (bounded) and writes NaN.  A warp whose wait was given up does not
+// arrive on the empty barriers: it runs ahead of the others, and two arrivals of a diagonal tile on a
+// barrier that waits for one are undefined.
 #include <algorithm>
 
 #include "sg_internal.h"
@@ -49,7 +49,7 @@ struct BlockArgs {
   int N, m, P, nb, rounds, ntile, ntiles_row, slots;
   long long item_elems;
   int evict_first;
-  long long wait_limit;  // polls after which a wait between the CTA's warps gives up
+  int fail;  // tests: start as if a wait had given up
 };
 
 template <typename T>
@@ -112,7 +112,8 @@ __global__ void __launch_bounds__((kBlockMaxWarps + 1) * 32) block_edge_kernel(
   for (int i = tid; i < g.rounds * nb; i += blockDim.x) tab[i] = table[i];
   for (int i = tid; i < g.ntile; i += blockDim.x) kinds[i] = tkind[i];
   if (tid == 0) {
-    s_fail[0] = s_fail[1] = 0;
+    s_fail[0] = g.fail;
+    s_fail[1] = 0;
     for (int s = 0; s < g.slots; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 2);
@@ -133,7 +134,7 @@ __global__ void __launch_bounds__((kBlockMaxWarps + 1) * 32) block_edge_kernel(
       bool ok = true;
       auto wait_room = [&](unsigned long long* bar, unsigned parity) {
         if (mbar_try_wait(bar, parity)) return true;
-        for (long long n = 0; n < g.wait_limit && !*vfail; ++n)
+        for (long long n = 0; n < kWaitLimit && !*vfail; ++n)
           if (mbar_try_wait(bar, parity)) return true;
         return false;
       };
@@ -195,10 +196,10 @@ __global__ void __launch_bounds__((kBlockMaxWarps + 1) * 32) block_edge_kernel(
   auto wait_tile = [&](unsigned c, int slot) {
     for (long long n = 0; (int)(issued - c) <= 0; ++n) {
       issued = *vissued;
-      if (n >= g.wait_limit || *vfail) return false;
+      if (n >= kWaitLimit || *vfail) return false;
     }
     __threadfence_block();
-    return mbar_wait_bounded(&full[slot], (c >> slot_log) & 1u, g.wait_limit);
+    return mbar_wait_bounded(&full[slot], (c >> slot_log) & 1u);
   };
   if (sizeof(T) == 4 && (int)blockIdx.x < nitems) fetch(blockIdx.x);
   for (int it = blockIdx.x; it < nitems; it += gridDim.x, base += (unsigned)g.ntile) {
@@ -581,7 +582,7 @@ int launch_block_op(const System& s, const BlockOp& op, const T* X, T* Y, T alph
   if (!op.ready || F == nullptr) return fail(SG_ERR_ARG, "block operator not built");
   const BlockArgs g{s.N, s.pat.m, s.P, op.nb, op.rounds, op.ntile, op.row_tiles, op.slots,
                     (long long)op.nval * kBR, op.bytes > ((size_t)64 << 20) ? 1 : 0,
-                    test_wait_limit()};
+                    test_block_fail()};
   auto kern = block_kernel<T>(op.TS);
   TimeScope ts(s.timer, sizeof(T) == 8 ? K_APPLY_F64 : K_APPLY_LOWP, st);
   SG_TRY(launch_pdl(kern, dim3(op.grid), dim3((op.nb + 1) * 32), op.smem, st, g, (const int*)op.table.p,

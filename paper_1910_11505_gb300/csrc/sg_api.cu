@@ -62,8 +62,8 @@ size_t smem_optin_max() {
 }
 
 // What the tests of failure paths set on their own thread (sg_test_hook).
-static thread_local long long g_test_wait = -1;
-long long test_wait_limit() { return g_test_wait >= 0 ? g_test_wait : kWaitLimit; }
+static thread_local int g_test_block_fail = 0;
+int test_block_fail() { return g_test_block_fail; }
 
 TimeScope::TimeScope(Timer* t_, int cls_, cudaStream_t st_) : t(t_), cls(cls_), st(st_) {
   if (!t || !t->on) return;
@@ -1342,11 +1342,11 @@ void sg_free(sg_handle* h) {
   delete h;
 }
 
-// For the tests of failure paths; acts on the calling thread alone.  what 0: polls after which the
-// block-stencil operator's waits give up (0: at once; negative: the usual limit).
+// For the tests of failure paths; acts on the calling thread alone.  what 0: value 1 has the CTAs of
+// the block-stencil operator start as if a wait had given up, 0 ends that.
 int sg_test_hook(int what, long long value) {
   if (what != 0) return fail(SG_ERR_ARG, "unknown hook");
-  g_test_wait = value;
+  g_test_block_fail = value != 0;
   return SG_OK;
 }
 

@@ -55,9 +55,9 @@ int launch_train_tc(int B, int h2, int out, const float* H2, const __nv_bfloat16
 size_t w3_tiles_elems(int out);
 int launch_w3_tiles(int out, int h2, const float* W3, __nv_bfloat16* W3c, cudaStream_t st);
 
-// Set by tests on their own thread (sg_test_hook in sg_api.cu): polls after which the waits of the
-// block-stencil operator give up (kWaitLimit unless set).
-long long test_wait_limit();
+// Set by tests on their own thread (sg_test_hook in sg_api.cu): the block-stencil operator's CTAs
+// start as if a wait had given up.
+int test_block_fail();
 
 // ------------------------------------------------------------------ live kernel timing
 
@@ -160,9 +160,8 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, unsigned 
 }
 
 // Bounded wait for the given phase parity of an mbarrier.
-__device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsigned parity,
-                                                  long long limit = kWaitLimit) {
-  for (long long it = 0; it < limit; ++it)
+__device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsigned parity) {
+  for (long long it = 0; it < kWaitLimit; ++it)
     if (mbar_try_wait(bar, parity)) return true;
   return false;
 }

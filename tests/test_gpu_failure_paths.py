@@ -18,9 +18,9 @@ def _hook(what, value):
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
 @pytest.mark.parametrize("n,M,p", [(40, 4, 3), (12, 6, 3), (60, 3, 2)])
 def test_block_operator_waits_that_give_up(n, M, p, precision):
-    # every wait between the kernel's warps gives up at its first poll: interior rows are NaN, boundary
-    # rows are X, the kernel ends, and the next call is right (several items per CTA, rings shorter and
-    # longer than an item's tiles, odd and even numbers of ranges)
+    # every CTA goes on as after a wait that was given up: interior rows are NaN, boundary rows are X, the
+    # kernel ends, and the next call is right (several items per CTA, rings shorter and longer than an
+    # item's tiles, odd and even numbers of ranges)
     h = sg.sg_setup(sg.sg_default_params(n=n, M=M, p=p, sigma=0.8, ell=0.6, precision=precision))
     assert sg.sg_op_info(h)[precision]["kernel"] == "block"
     prob = O.build_problem(n, M, p, sigma=0.8, ell=0.6)
@@ -29,11 +29,11 @@ def test_block_operator_waits_that_give_up(n, M, p, precision):
     X = torch.from_numpy(W.random_field(prob.N, prob.P, seed=3)).cuda().to(dt)
     Y = torch.zeros_like(X)
     try:
-        _hook(0, 0)
+        _hook(0, 1)
         apply(h, 0, X, Y)
         torch.cuda.synchronize()
     finally:
-        _hook(0, -1)
+        _hook(0, 0)
     inner = torch.zeros(n + 1, n + 1, dtype=torch.bool, device="cuda")
     inner[1:-1, 1:-1] = True
     inner = inner.reshape(-1)
