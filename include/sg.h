@@ -154,11 +154,14 @@ int sg_nnz(const sg_handle* h, int sys, long long* nnz_A, long long* nnz_G);
 /* Y = K X = sum_k A_k X G_k^T (Eqs. stochastic_matrix, K_matrix); X, Y device, N x P FP64,
  * must not overlap.  Asynchronous on ``stream``.  Calls on several streams may overlap: what the
  * block-stencil operator stores between its two kernels comes from the handle's memory pool in
- * stream order (a call under capture adds an allocation and a free node to the graph). */
+ * stream order.  A call under capture takes a block of its own (5 N P values), which the graph holds
+ * until it and its instances are destroyed; sg_free takes all blocks, so call it after the last
+ * replay. */
 int sg_matvec(sg_handle* h, int sys, const double* X, double* Y, void* stream);
 
-/* Same operator with the FP32 (precision SG_MIXED_FP32) or BF16 (SG_MIXED_BF16) copy of the
- * stiffness stack and FP32 arithmetic; X, Y device N x P FP32.  SG_ERR_ARG for an FP64 system. */
+/* Same operator (also as to streams and capture) with the FP32 (precision SG_MIXED_FP32) or BF16
+ * (SG_MIXED_BF16) copy of the stiffness stack and FP32 arithmetic; X, Y device N x P FP32.
+ * SG_ERR_ARG for an FP64 system. */
 int sg_matvec_lowp(sg_handle* h, int sys, const float* X, float* Y, void* stream);
 
 /* Z = P^{-1} R for the system's preconditioner, with ``outer_sweeps`` steps of Eq. level_solver

@@ -762,8 +762,70 @@ static int make_pool(sg_handle* h, cudaStream_t st) {
   return SG_OK;
 }
 
+// A captured call's scratch.  Allocation nodes in the graph would keep it from being a child graph or
+// having two instances; a block of the handle has no such rules.  The graph holds a user object whose
+// end (with the graph's last instance) gives the block back for the next capture.  Every call has its
+// own: two instances that run at the same time then write the same values to it, as they do to Y.
+struct CaptureRef {
+  std::shared_ptr<CaptureStore> store;
+  size_t index;
+};
+static void CUDART_CB release_captured(void* arg) {
+  CaptureRef* r = static_cast<CaptureRef*>(arg);
+  {
+    std::lock_guard<std::mutex> lock(r->store->mu);
+    if (r->index < r->store->blocks.size()) r->store->blocks[r->index].held = false;
+  }
+  delete r;
+}
+
+// Null if there is no memory for it.
+static void* captured_scratch(sg_handle* h, size_t bytes, cudaGraph_t graph) {
+  CaptureStore& c = *h->captured;
+  std::lock_guard<std::mutex> lock(c.mu);
+  size_t at = c.blocks.size();
+  for (size_t i = 0; i < c.blocks.size(); ++i)  // the smallest free one that is large enough
+    if (!c.blocks[i].held && c.blocks[i].bytes >= bytes &&
+        (at == c.blocks.size() || c.blocks[i].bytes < c.blocks[at].bytes))
+      at = i;
+  if (at == c.blocks.size()) {
+    void* p = nullptr;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // allows cudaMalloc on this thread
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t e = cudaMalloc(&p, bytes);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    c.blocks.push_back({p, bytes, false});
+  }
+  CaptureRef* ref = new CaptureRef{h->captured, at};
+  cudaUserObject_t obj;
+  if (cudaUserObjectCreate(&obj, ref, release_captured, 1, cudaUserObjectNoDestructorSync) != cudaSuccess) {
+    delete ref;
+    cudaGetLastError();
+    return nullptr;
+  }
+  c.blocks[at].held = true;
+  if (cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+    cudaUserObjectRelease(obj, 1);  // (its end marks the block free)
+    cudaGetLastError();
+    return nullptr;
+  }
+  return c.blocks[at].p;
+}
+
 template <typename T, typename Run, typename Pairs>
 static int matvec_pooled(sg_handle* h, System& s, cudaStream_t st, Run run, Pairs pairs) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &status) != cudaSuccess) cudaGetLastError();
+  if (status == cudaStreamCaptureStatusActive) {
+    cudaGraph_t graph = nullptr;
+    SG_CUDA(cudaStreamGetCaptureInfo(st, &status, nullptr, &graph, nullptr, nullptr, nullptr));
+    void* f = captured_scratch(h, sizeof(T) * block_scratch_elems(s), graph);
+    return f != nullptr ? run((T*)f) : pairs();
+  }
   void* p = nullptr;
   if (cudaMallocFromPoolAsync(&p, sizeof(T) * block_scratch_elems(s), h->pool, st) != cudaSuccess) {
     cudaGetLastError();  // no memory for another stream's products: the kernel that needs none
@@ -1339,6 +1401,11 @@ void sg_free(sg_handle* h) {
   for (auto* s : h->sys) free_system(s);
   for (auto& e : h->timer.ev) cudaEventDestroy(e);
   if (h->pool) cudaMemPoolDestroy(h->pool);
+  {
+    std::lock_guard<std::mutex> lock(h->captured->mu);
+    for (auto& b : h->captured->blocks) cudaFree(b.p);
+    h->captured->blocks.clear();
+  }
   delete h;
 }
 

@@ -5,6 +5,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -479,12 +481,25 @@ struct System {
   DBuf<int> mg_nodes;
 };
 
+// Scratch of the sg_matvec calls of captured graphs: a block for every call, held until the graph
+// and its instances are gone.
+struct CaptureStore {
+  struct Block {
+    void* p;
+    size_t bytes;
+    bool held;
+  };
+  std::mutex mu;
+  std::vector<Block> blocks;
+};
+
 }  // namespace sg
 
 struct sg_handle {
   std::vector<sg::System*> sys;
   int device = 0;
   cudaMemPool_t pool = nullptr;  // scratch of sg_matvec calls (block-stencil operator), by stream
+  std::shared_ptr<sg::CaptureStore> captured = std::make_shared<sg::CaptureStore>();
   sg::Timer timer;
 };
 
