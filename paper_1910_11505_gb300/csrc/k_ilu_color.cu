@@ -9,6 +9,8 @@
 // has a lower colour hold the unit lower factor l_ij, slots of a higher colour hold u_ij / u_ii,
 // slot 4 holds 1 / u_ii.
 #include <algorithm>
+#include <map>
+#include <mutex>
 
 #include "sg_internal.h"
 
@@ -689,8 +691,8 @@ template <typename T>
 using ClusterKern = void (*)(int, int, int, int, int, int, const int*, const T*, T*, T*, const int*,
                              const T*, T*);
 
-// Whether clusters of 16 CTAs of 1024 threads (a non-portable size) can be scheduled on this
-// device: asked once per process and kernel; on any failure the answer is no.
+// Whether clusters of 16 CTAs of 1024 threads (a non-portable size) can be scheduled on the current
+// device, and the attributes that allow them there; on any failure the answer is no.
 template <typename T>
 bool cluster16_ok(ClusterKern<T> kern, size_t smem) {
   bool ok = false;
@@ -820,12 +822,22 @@ template int launch_color_gs<float, __nv_bfloat16>(System&, int, const float*, f
                                                    const int*, const float*, float*,
                                                    const __nv_bfloat16*, const float*);
 
-// The largest split form whose 16 CTAs are asked for is the largest that fits.
+// Asked once per device (a kernel's attributes are set for each).  The largest split form whose 16
+// CTAs are asked for is the largest that fits.
 template <typename T>
 static bool clusters16(int m, bool in_smem) {
-  static const bool split = cluster16_ok<T>(color_split_kernel<T, 16>, kColorSmemMax);
-  static const bool plain = cluster16_ok<T>(color_cluster_kernel<T, 16>, 0);
-  return in_smem && split_smem<T>(m, 16) > 0 ? split : plain;
+  static std::mutex mu;
+  static std::map<int, std::pair<bool, bool>> known;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lock(mu);
+  auto it = known.find(dev);
+  if (it == known.end()) {
+    const bool split = cluster16_ok<T>(color_split_kernel<T, 16>, kColorSmemMax);
+    const bool plain = cluster16_ok<T>(color_cluster_kernel<T, 16>, 0);
+    it = known.emplace(dev, std::make_pair(split, plain)).first;
+  }
+  return in_smem && split_smem<T>(m, 16) > 0 ? it->second.first : it->second.second;
 }
 
 // Block solves of columns a0 .. a0 + ncols - 1 from Rt into Z (colour-ordered factors).
