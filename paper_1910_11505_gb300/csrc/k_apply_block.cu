@@ -436,6 +436,20 @@ size_t block_smem(const BlockPlan& pl, int elem, int slots) {
          (size_t)pl.nb * pl.TS * kBLd * elem;
 }
 
+// Ring slots, a power of two.  CTAs per SM so that about 28 warps are resident (12 ranges of fields:
+// 2, 5: 4, 3: 7), their rings sharing some 200 KB; one that is alone on its SM (from 14 ranges on)
+// has to fit its differences and tables beside the ring (FP64 P = 126, 18 ranges: 8 slots, not 16;
+// n = 24 144 us against the pair kernel's 1060).  0 where two slots do not fit.
+int block_slots(const BlockPlan& pl, int elem) {
+  const size_t slot = (size_t)pl.TS * pl.TS * kBR * elem;
+  const size_t want = (200 * 1024) / std::max(1, std::min(8, 28 / (pl.nb + 1)));
+  const size_t most = smem_optin_max();
+  int slots = 2;
+  if (block_smem(pl, elem, slots) > most) return 0;
+  while (slots < 32 && 2 * slots * slot <= want && block_smem(pl, elem, 2 * slots) <= most) slots *= 2;
+  return slots;
+}
+
 template <typename T>
 void (*block_kernel(int ts))(BlockArgs, const int*, const int*, const T*, const T*, T*, const int*, int*) {
   switch (ts) {
@@ -474,7 +488,7 @@ size_t block_scratch_elems(const System& s) { return (size_t)kBlockEdges * s.N *
 // P >= 10 or 300 k values.
 size_t block_op_bytes(const System& s, int elem) {
   BlockPlan pl;
-  if (s.pat.m < 4 || !plan_block(s.P, pl)) return 0;
+  if (s.pat.m < 4 || !plan_block(s.P, pl) || block_slots(pl, elem) == 0) return 0;
   if ((unsigned long long)s.N * (unsigned long long)s.P >= (1ull << 31)) return 0;
   if (sizeof(double) * (size_t)s.L * 9 > smem_optin_max()) return 0;
   const size_t tiles = ((size_t)s.N - 2 * (s.pat.m + 1) + kBR - 1) / kBR;
@@ -493,14 +507,8 @@ int build_block_op(System& s, BlockOp& op, int elem, cudaStream_t st) {
   op.ntile = pl.ntile;
   op.nval = pl.nval;
   op.row_tiles = (s.N - 2 * (s.pat.m + 1) + kBR - 1) / kBR;
-  // CTAs per SM so that about 28 warps are resident (12 ranges of fields: 2, 5: 4, 3: 7), their
-  // rings sharing some 200 KB; a power of two of slots
-  const size_t slot = (size_t)pl.TS * pl.TS * kBR * elem;
-  const size_t want = (200 * 1024) / std::max(1, std::min(8, 28 / (pl.nb + 1)));
-  op.slots = 2;
-  while (op.slots < 32 && 2 * op.slots * slot <= want) op.slots *= 2;
+  op.slots = block_slots(pl, elem);
   op.smem = block_smem(pl, elem, op.slots);
-  if (op.smem > smem_optin_max()) return fail(SG_ERR_ARG, "block operator: shared memory");
   // triples of every value
   std::vector<std::vector<std::pair<int, double>>> per((size_t)s.P * s.P);
   for (const Triple& t : s.triples)
