@@ -86,11 +86,13 @@ typedef struct {
   int mg_coarse;     /* SG_PC_MG: cells per side of the coarsest mesh (the paper: 2); n must be  */
                      /* mg_coarse times a power of two, and the coarsest interior system of     */
                      /* (mg_coarse - 1)^2 P unknowns is solved with its dense inverse (<= 4096)  */
-  int op_kernel;     /* SG operator kernel: SG_OP_AUTO (the block-stencil operator while its     */
-                     /* assembled blocks take at most an eighth of the device memory and leave   */
-                     /* half of it free; else time the other candidates on this system at setup  */
-                     /* and keep the fastest, cached per N, P, L and precision for the process), */
-                     /* SG_OP_PAIRS or SG_OP_TILE                                               */
+  int op_kernel;     /* SG operator kernel: SG_OP_AUTO, SG_OP_PAIRS or SG_OP_TILE.  AUTO takes the   */
+                     /* block-stencil operator while its assembled blocks take at most an eighth */
+                     /* of the device memory and leave half of it free, unless a coefficient    */
+                     /* degree q < 2p makes the sparse kernels' work less than twice its own:    */
+                     /* then, and where there is no room, it times the candidates on this system */
+                     /* at setup and keeps the fastest, cached per N, P, L, q and precision for  */
+                     /* the process.  The forms agree to rounding.                               */
   int op_kappa;      /* SG_OP_TILE: k per register group, 1, 2 or 4 (0: 2 in FP64, 4 in FP32)   */
   int op_ctas;       /* SG_OP_TILE: CTAs per SM the shared memory is planned for, 1 or 2 (0: 1) */
   int ilu_order;     /* ILU(0) node ordering: SG_ILU_NATURAL, or SG_ILU_COLOR4 (colour           */

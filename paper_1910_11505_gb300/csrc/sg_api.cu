@@ -258,8 +258,10 @@ int host_tables(System& s) {
 
 // ------------------------------------------------------------------ operator kernel tuner
 
-// The choice for one system shape and operator precision: the pair kernel, or the row-tiled kernel
-// with kappa k per register group and shared memory planned for ``ctas`` CTAs per SM.
+// The choice for one system shape and operator precision: the pair kernel, the row-tiled kernel
+// with kappa k per register group and shared memory planned for ``ctas`` CTAs per SM, or the
+// block-stencil operator.
+constexpr int kOpBlock = -1;
 struct TuneChoice {
   int kernel = SG_OP_PAIRS, kappa = 0, ctas = 1;
   double ms = 0.0;
@@ -269,6 +271,7 @@ static std::map<std::array<long long, 5>, TuneChoice> g_tune;
 
 static std::string describe(const TuneChoice& c) {
   if (c.kernel == SG_OP_PAIRS) return "pairs";
+  if (c.kernel == kOpBlock) return "block";
   return "tile k" + std::to_string(c.kappa) + " x" + std::to_string(c.ctas);
 }
 
@@ -284,8 +287,11 @@ static size_t smem_budget(int ctas) {
   return std::min(opt, each > 1024 ? each - 1024 : each);
 }
 
+// Milliseconds of one application among others (*ms); with ``flush``, a buffer larger than L2, plus
+// those of one whose operands are all in memory.
 template <typename T>
-static int time_operator(const System& s, const T* X, T* Y, cudaStream_t st, double* ms) {
+static int time_operator(const System& s, const T* X, T* Y, cudaStream_t st, const DBuf<unsigned char>* flush,
+                         double* ms) {
   auto run = [&]() {
     if constexpr (sizeof(T) == 8) return launch_matvec_f64(s, X, Y, 1.0, nullptr, 0.0, st);
     else return launch_matvec_f32(s, X, Y, 1.0f, nullptr, 0.0f, st);
@@ -294,21 +300,31 @@ static int time_operator(const System& s, const T* X, T* Y, cudaStream_t st, dou
   SG_CUDA(cudaEventCreate(&a));
   SG_CUDA(cudaEventCreate(&b));
   int rc = run();
-  if (rc == SG_OK) rc = cudaEventRecord(a, st) == cudaSuccess ? SG_OK : SG_ERR_CUDA;
-  for (int r = 0; r < 3 && rc == SG_OK; ++r) rc = run();
-  if (rc == SG_OK) rc = cudaEventRecord(b, st) == cudaSuccess ? SG_OK : SG_ERR_CUDA;
-  float t = 0.f;
-  if (rc == SG_OK && cudaEventSynchronize(b) == cudaSuccess && cudaEventElapsedTime(&t, a, b) == cudaSuccess)
-    *ms = t / 3.0;
-  else if (rc == SG_OK)
-    rc = fail(SG_ERR_CUDA, "timing the operator failed");
+  *ms = 0.0;
+  for (int pass = 0; pass < (flush ? 4 : 1) && rc == SG_OK; ++pass) {  // three runs in a row, three alone
+    if (pass > 0 && cudaMemsetAsync(flush->p, 0, flush->n, st) != cudaSuccess) rc = SG_ERR_CUDA;
+    if (rc == SG_OK) rc = cudaEventRecord(a, st) == cudaSuccess ? SG_OK : SG_ERR_CUDA;
+    for (int r = 0; r < (pass > 0 ? 1 : 3) && rc == SG_OK; ++r) rc = run();
+    if (rc == SG_OK) rc = cudaEventRecord(b, st) == cudaSuccess ? SG_OK : SG_ERR_CUDA;
+    float t = 0.f;
+    if (rc == SG_OK && cudaEventSynchronize(b) == cudaSuccess && cudaEventElapsedTime(&t, a, b) == cudaSuccess)
+      *ms += t / 3.0;
+    else if (rc == SG_OK)
+      rc = fail(SG_ERR_CUDA, "timing the operator failed");
+  }
   cudaEventDestroy(a);
   cudaEventDestroy(b);
   return rc;
 }
 
-// Whether the block-stencil operator is to serve this system in precision ``elem``: it takes more
-// memory than the row-tiled one (2 to 4 times its stack), so it is kept to an eighth of the
+static int current_device() {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  return dev;
+}
+
+// Whether there is room for the block-stencil operator of this system in precision ``elem``: it takes
+// more memory than the row-tiled one (2 to 4 times its stack), so it is kept to an eighth of the
 // device's memory and to the half of it that is left free otherwise.
 static bool block_op_wanted(const System& s, int elem) {
   const size_t bytes = block_op_bytes(s, elem);
@@ -321,47 +337,73 @@ static bool block_op_wanted(const System& s, int elem) {
   return bytes <= total_b / 8 && free_b >= bytes + total_b / 2;
 }
 
+// The block-stencil operator does 5 P^2 multiply-adds and streams 5 P (P + 1) / 2 values a node whatever
+// the coefficient is; the sparse forms do 9 U + nnz_G (U pairs (k, b) that meet a triple product).
+// At q = 2 p that is at least 2.2 times as many (P = 84: 3.3) and the block form takes 0.2 to 0.6 of
+// their time, so from a factor of 2 on nothing is timed.  Low coefficient degrees turn it round: below
+// a quarter the block form lost at every size (M = 6, p = 3, q = 1, factor 0.11: n = 256 FP32 753
+// against 121 us, FP64 4.23 against 0.77 ms; M = 4, p = 3, q = 1, 0.22: n = 256 FP64 759 against 261, n =
+// 48 FP32 11.4 against 10.2).  Between them size and precision decide (M = 6, p = 3, q = 3, 0.85: n = 97
+// FP32 111 against 74 us, n = 24 21 against 46, n = 256 FP64 4.23 against 4.86 ms), so all are timed.
+constexpr double kBlockAlways = 2.0, kBlockNever = 0.25;
+// A sparse form has to be this much faster than the block form to be kept, so that two setups of a
+// system whose forms are close do not differ.
+constexpr double kBlockMargin = 0.9;
+
 // Build the operator kernel of precision ``elem`` (8: FP64, 4: FP32) that op_kernel asks for.
-// SG_OP_AUTO times the pair kernel and every row-tiled variant that fits (kappa 1, 2, 4; one or
-// two CTAs per SM) on this system, keeps the fastest and caches the choice for the system's
-// (N, P, L, q, element size).
-static int choose_operator(System& s, int elem, cudaStream_t st) {
+// SG_OP_AUTO takes the block-stencil operator where the counts above favour it; else it times the pair
+// kernel, every row-tiled variant that fits (kappa 1, 2, 4; one or two CTAs per SM) and, unless the
+// counts rule it out, the block-stencil operator on this system, keeps the fastest and caches the
+// choice for the system's (N, P, L, q, element size).  Sparse forms are timed among one another in a
+// row; against the block form, whose values may or may not stay in L2 between the applications of
+// a program, in a row and alone.
+static int choose_operator(System& s, int elem, cudaStream_t st, bool allow_block = true) {
   TileOp& op = elem == 8 ? s.tile64 : s.tile32;
+  BlockOp& blk = elem == 8 ? s.block64 : s.block32;
   const sg_params& p = s.prm;
   std::string& note = s.tile_msg;
+  const std::string prec = elem == 8 ? "fp64: " : "fp32: ";
   if (p.op_kernel == SG_OP_PAIRS) return SG_OK;
-  if (p.op_kernel == SG_OP_AUTO && block_op_wanted(s, elem)) {
-    BlockOp& blk = elem == 8 ? s.block64 : s.block32;
+  const double share = (9.0 * s.op.npairs + s.op.nent) / (5.0 * s.P * s.P);
+  bool block = allow_block && p.op_kernel == SG_OP_AUTO && share >= kBlockNever && block_op_bytes(s, elem) > 0;
+  if (block && !block_op_wanted(s, elem)) {
+    note += prec + "no memory for block; ";
+    block = false;
+  }
+  // SG_OK; or, without memory for it, the choice among the other forms
+  auto build_block = [&](const std::string& how) {
     const int rc = build_block_op(s, blk, elem, st);
     if (rc == SG_OK) {
-      const std::array<long long, 5> key{s.N, s.P, s.L, p.q, -elem};
-      std::lock_guard<std::mutex> lock(g_tune_mu);
-      note += std::string(elem == 8 ? "fp64" : "fp32") +
-              (g_tune.count(key) ? ": block (cached); " : ": chose block; ");
-      g_tune[key] = TuneChoice();
-      return SG_OK;
+      note += prec + "block" + how + "; ";
+      return rc;
     }
     free_block_op(blk);
-    if (rc != SG_ERR_ARG && rc != SG_ERR_OOM) return rc;
+    if (rc != SG_ERR_OOM && rc != SG_ERR_ARG) return rc;
+    note += prec + "no block (" + g_last_error + "); ";
     set_error("");
-  }
+    return choose_operator(s, elem, st, false);
+  };
+  if (block && share >= kBlockAlways) return build_block("");
   if (p.op_kernel == SG_OP_TILE) {
     const int kappa = p.op_kappa ? p.op_kappa : (elem == 8 ? 2 : 4);
     const int ctas = p.op_ctas ? p.op_ctas : 1;
     if (build_tile_op(s, op, kappa, elem, smem_budget(ctas), st, ctas) != SG_OK) {
-      note += (elem == 8 ? "fp64: " : "fp32: ") + g_last_error + "; ";
+      note += prec + g_last_error + "; ";
       free_tile_op(op);
       set_error("");
     }
     return SG_OK;
   }
-  const std::array<long long, 5> key{s.N, s.P, s.L, p.q, elem};
+  // choices among all forms and among the sparse ones are kept apart
+  const std::array<long long, 5> key{s.N, s.P, s.L, p.q, block ? -elem : elem};
   {
-    std::lock_guard<std::mutex> lock(g_tune_mu);
+    std::unique_lock<std::mutex> lock(g_tune_mu);
     auto itc = g_tune.find(key);
     if (itc != g_tune.end()) {
       const TuneChoice c = itc->second;
-      note += std::string(elem == 8 ? "fp64: " : "fp32: ") + describe(c) + " (cached); ";
+      lock.unlock();
+      if (c.kernel == kOpBlock) return build_block(" (cached)");
+      note += prec + describe(c) + " (cached); ";
       if (c.kernel == SG_OP_PAIRS) return SG_OK;
       if (build_tile_op(s, op, c.kappa, elem, smem_budget(c.ctas), st, c.ctas) != SG_OK) {
         free_tile_op(op);
@@ -371,18 +413,33 @@ static int choose_operator(System& s, int elem, cudaStream_t st) {
     }
   }
   const size_t NP = (size_t)s.N * s.P;
-  DBuf<unsigned char> xb, yb;
-  SG_TRY(xb.alloc(NP * elem));
-  SG_TRY(yb.alloc(NP * elem));
-  SG_CUDA(cudaMemsetAsync(xb.p, 0, NP * elem, st));
+  struct Bufs {  // released on every way out
+    DBuf<unsigned char> x, y, flush;
+    ~Bufs() {
+      x.release();
+      y.release();
+      flush.release();
+    }
+  } b;
+  SG_TRY(b.x.alloc(NP * elem));
+  SG_TRY(b.y.alloc(NP * elem));
+  SG_CUDA(cudaMemsetAsync(b.x.p, 0, NP * elem, st));
+  const DBuf<unsigned char>* flush = nullptr;
+  if (block) {  // (without memory for the flush, in a row alone)
+    int l2 = 0;
+    if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, current_device()) == cudaSuccess && l2 > 0 &&
+        b.flush.alloc(2 * (size_t)l2) == SG_OK)
+      flush = &b.flush;
+    set_error("");
+  }
   auto timed = [&](double* ms) {
     if (elem == 8)
-      return time_operator<double>(s, (const double*)xb.p, (double*)yb.p, st, ms);
-    return time_operator<float>(s, (const float*)xb.p, (float*)yb.p, st, ms);
+      return time_operator<double>(s, (const double*)b.x.p, (double*)b.y.p, st, flush, ms);
+    return time_operator<float>(s, (const float*)b.x.p, (float*)b.y.p, st, flush, ms);
   };
   TuneChoice best;
   std::string log = std::string(elem == 8 ? "fp64:" : "fp32:");
-  SG_TRY(timed(&best.ms));  // the pair kernel (no row-tiled operator built yet)
+  SG_TRY(timed(&best.ms));  // the pair kernel (no other operator built yet)
   log += " pairs " + std::to_string(best.ms) + " ms";
   for (int ctas : {1, 2})
     for (int kappa : {1, 2, 4}) {
@@ -407,8 +464,25 @@ static int choose_operator(System& s, int elem, cudaStream_t st) {
       free_tile_op(cand);
       set_error("");
     }
-  xb.release();
-  yb.release();
+  if (block) {
+    double ms = 0.0;
+    const int rc = build_block_op(s, blk, elem, st);
+    if (rc == SG_OK && timed(&ms) == SG_OK) {
+      log += ", block " + std::to_string(ms) + " ms";
+      if (best.ms >= kBlockMargin * ms) {
+        best = TuneChoice{kOpBlock, 0, 0, ms};
+        free_tile_op(op);
+      }
+    }
+    if (best.kernel != kOpBlock) free_block_op(blk);
+    if (rc != SG_OK && rc != SG_ERR_OOM && rc != SG_ERR_ARG) return rc;
+    if (rc != SG_OK) {  // nothing is learned for setups that have the memory
+      note += log + "; no block (" + g_last_error + "); ";
+      set_error("");
+      return SG_OK;
+    }
+    set_error("");
+  }
   note += log + "; chose " + describe(best) + "; ";
   std::lock_guard<std::mutex> lock(g_tune_mu);
   g_tune[key] = best;
