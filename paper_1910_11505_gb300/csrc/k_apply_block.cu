@@ -379,7 +379,7 @@ struct BlockPlan {
 
 // Range size with the fewest padded values (the larger one on a tie: fewer reads of d per value),
 // among those that leave at most kBlockMaxWarps ranges.
-bool plan_block(int P, BlockPlan& pl) {
+bool plan_sizes(int P, BlockPlan& pl) {
   long long best = -1;
   for (int ts : {4, 5, 6, 7}) {
     const int nb = (P + ts - 1) / ts;
@@ -393,8 +393,13 @@ bool plan_block(int P, BlockPlan& pl) {
   }
   if (best < 0) return false;
   pl.nval = (int)best;
+  pl.rounds = pl.nb;  // odd: each with one diagonal tile; even: nb - 1 of pairs and one of diagonals
+  pl.ntile = pl.nb * (pl.nb + 1) / 2;
+  return true;
+}
+
+void plan_tables(BlockPlan& pl) {
   const int nb = pl.nb, odd = nb & 1, n = odd ? nb : nb - 1;
-  pl.rounds = nb;  // odd: each with one diagonal tile; even: nb - 1 of pairs and one of diagonals
   pl.table.assign((size_t)pl.rounds * nb, 0);
   int s = 0;
   auto put = [&](int r, int a, int b) {
@@ -426,8 +431,6 @@ bool plan_block(int P, BlockPlan& pl) {
     }
   if (!odd)
     for (int a = 0; a < nb; ++a) put(nb - 1, a, a);
-  pl.ntile = s;
-  return true;
 }
 
 size_t block_smem(const BlockPlan& pl, int elem, int slots) {
@@ -471,13 +474,6 @@ int run_assemble(const System& s, const BlockOp& op, const int* vptr, const int*
   return check_launch("block_assemble");
 }
 
-template <typename T>
-T* block_store(const BlockOp& op);
-template <>
-double* block_store<double>(const BlockOp& op) { return op.k64.p; }
-template <>
-float* block_store<float>(const BlockOp& op) { return op.k32.p; }
-
 }  // namespace
 
 size_t block_scratch_elems(const System& s) { return (size_t)kBlockEdges * s.N * s.P; }
@@ -488,7 +484,7 @@ size_t block_scratch_elems(const System& s) { return (size_t)kBlockEdges * s.N *
 // P >= 10 or 300 k values.
 size_t block_op_bytes(const System& s, int elem) {
   BlockPlan pl;
-  if (s.pat.m < 4 || !plan_block(s.P, pl) || block_slots(pl, elem) == 0) return 0;
+  if (s.pat.m < 4 || !plan_sizes(s.P, pl) || block_slots(pl, elem) == 0) return 0;
   if ((unsigned long long)s.N * (unsigned long long)s.P >= (1ull << 31)) return 0;
   if (sizeof(double) * (size_t)s.L * 9 > smem_optin_max()) return 0;
   const size_t tiles = ((size_t)s.N - 2 * (s.pat.m + 1) + kBR - 1) / kBR;
@@ -496,10 +492,16 @@ size_t block_op_bytes(const System& s, int elem) {
   return tiles * kBlockEdges * (size_t)pl.nval * kBR * elem;
 }
 
+// One allocation holds the tiles, the products of an application, and the tables (those of the
+// assembly too), which one copy brings, and a mixed system's FP32 tiles are the FP64 ones rounded.
+// Bound: allocations and copies, each of which waits for the stream, on small meshes; the assembly's
+// multiply-adds on large ones.  Setup of 64 systems of 64 x 64 (P = 35, five levels) 1.69 -> 1.59 s, of
+// one of 256 x 256 (P = 84, FP32) 219 -> 206 ms, against ten allocations, five copies and two assemblies.
 int build_block_op(System& s, BlockOp& op, int elem, cudaStream_t st) {
   BlockPlan pl;
-  if (block_op_bytes(s, elem) == 0 || !plan_block(s.P, pl))
+  if (block_op_bytes(s, elem) == 0 || !plan_sizes(s.P, pl))
     return fail(SG_ERR_ARG, "block operator: unsupported sizes");
+  plan_tables(pl);
   op.elem = elem;
   op.TS = pl.TS;
   op.nb = pl.nb;
@@ -509,58 +511,57 @@ int build_block_op(System& s, BlockOp& op, int elem, cudaStream_t st) {
   op.row_tiles = (s.N - 2 * (s.pat.m + 1) + kBR - 1) / kBR;
   op.slots = block_slots(pl, elem);
   op.smem = block_smem(pl, elem, op.slots);
-  // triples of every value
-  std::vector<std::vector<std::pair<int, double>>> per((size_t)s.P * s.P);
+  // triples of every field pair a <= b, in k order, then of every value
+  const auto pair_of = [&](const Triple& t) { return (size_t)t.a * s.P + t.b; };
+  std::vector<int> first((size_t)s.P * s.P + 1, 0);
   for (const Triple& t : s.triples)
-    if (t.a <= t.b) per[(size_t)t.a * s.P + t.b].push_back({t.k, t.g});
-  std::vector<int> vptr(1, 0), vk;
-  std::vector<double> vg;
+    if (t.a <= t.b) ++first[pair_of(t) + 1];
+  for (size_t i = 1; i < first.size(); ++i) first[i] += first[i - 1];
+  std::vector<const Triple*> order(first.back());
+  std::vector<int> next(first.begin(), first.end() - 1);
+  for (const Triple& t : s.triples)
+    if (t.a <= t.b) order[next[pair_of(t)]++] = &t;
+  // tables: vg; then as ints table, tkind, the error word, vptr, vk
+  const size_t nent = order.size(), ntab = pl.table.size();
+  std::vector<double> host(nent + (ntab + pl.ntile + 1 + (pl.nval + 1) + nent + 1) / 2, 0.0);
+  int* const ints = reinterpret_cast<int*>(host.data() + nent);
+  std::copy(pl.table.begin(), pl.table.end(), ints);
+  std::copy(pl.tkind.begin(), pl.tkind.end(), ints + ntab);
+  int* const vptr = ints + ntab + pl.ntile + 1;
+  int* const vk = vptr + pl.nval + 1;
+  int q = 0;
   for (int v = 0; v < pl.nval; ++v) {
     const int a = pl.va[v], b = pl.vb[v];
-    if (a < s.P && b < s.P)
-      for (auto& e : per[(size_t)a * s.P + b]) {
-        vk.push_back(e.first);
-        vg.push_back(e.second);
+    if (a < s.P && b < s.P) {
+      const size_t i = (size_t)a * s.P + b;
+      for (int e = first[i]; e < first[i + 1]; ++e, ++q) {
+        host[q] = order[e]->g;
+        vk[q] = order[e]->k;
       }
-    vptr.push_back((int)vk.size());
-  }
-  DBuf<int> dptr, dk;
-  DBuf<double> dg;
-  struct Drop {  // the tables live until the assembly has run, on every way out
-    DBuf<int>&a, &b;
-    DBuf<double>& c;
-    ~Drop() {
-      a.release();
-      b.release();
-      c.release();
     }
-  } drop{dptr, dk, dg};
-  SG_TRY(dptr.alloc(vptr.size()));
-  SG_TRY(dptr.upload(vptr, st));
-  SG_TRY(dk.alloc(vk.size()));
-  SG_TRY(dk.upload(vk, st));
-  SG_TRY(dg.alloc(vg.size()));
-  SG_TRY(dg.upload(vg, st));
-  SG_TRY(op.table.alloc(pl.table.size()));
-  SG_TRY(op.table.upload(pl.table, st));
-  SG_TRY(op.tkind.alloc(pl.tkind.size()));
-  SG_TRY(op.tkind.upload(pl.tkind, st));
-  SG_TRY(op.err.alloc(1));
-  SG_CUDA(cudaMemsetAsync(op.err.p, 0, sizeof(int), st));
-  const size_t total = (size_t)op.row_tiles * kBlockEdges * pl.nval * kBR;
-  const bool wide = sizeof(double) * (size_t)s.L * 17 > smem_optin_max();
-  if (elem == 8) {
-    SG_TRY(op.f64.alloc(block_scratch_elems(s)));
-    SG_TRY(op.k64.alloc(total));
-    SG_TRY(wide ? (run_assemble<double, 8>(s, op, dptr.p, dk.p, dg.p, op.k64.p, st))
-                : (run_assemble<double, 16>(s, op, dptr.p, dk.p, dg.p, op.k64.p, st)));
-  } else {
-    SG_TRY(op.f32.alloc(block_scratch_elems(s)));
-    SG_TRY(op.k32.alloc(total));
-    SG_TRY(wide ? (run_assemble<float, 8>(s, op, dptr.p, dk.p, dg.p, op.k32.p, st))
-                : (run_assemble<float, 16>(s, op, dptr.p, dk.p, dg.p, op.k32.p, st)));
+    vptr[v + 1] = q;
   }
-  SG_CUDA(cudaStreamSynchronize(st));
+  const size_t total = (size_t)op.row_tiles * kBlockEdges * pl.nval * kBR;
+  const size_t scratch = (block_scratch_elems(s) * elem + 15) & ~(size_t)15;
+  SG_TRY(op.mem.alloc(total * elem + scratch + host.size() * sizeof(double)));
+  op.k = op.mem.p;
+  op.f = op.mem.p + total * elem;
+  double* const dg = reinterpret_cast<double*>(op.mem.p + total * elem + scratch);
+  op.table = reinterpret_cast<int*>(dg + nent);
+  op.tkind = op.table + ntab;
+  op.err = op.tkind + pl.ntile;
+  const int *dptr = op.err + 1, *dk = dptr + pl.nval + 1;
+  SG_CUDA(cudaMemcpyAsync(dg, host.data(), host.size() * sizeof(double), cudaMemcpyHostToDevice, st));
+  const bool wide = sizeof(double) * (size_t)s.L * 17 > smem_optin_max();
+  if (elem == 8)
+    SG_TRY(wide ? (run_assemble<double, 8>(s, op, dptr, dk, dg, (double*)op.k, st))
+                : (run_assemble<double, 16>(s, op, dptr, dk, dg, (double*)op.k, st)));
+  else if (s.block64.ready)  // the values of the FP64 operator, rounded (the same tiles)
+    SG_TRY(launch_cast_f32((const double*)s.block64.k, (float*)op.k, total, st));
+  else
+    SG_TRY(wide ? (run_assemble<float, 8>(s, op, dptr, dk, dg, (float*)op.k, st))
+                : (run_assemble<float, 16>(s, op, dptr, dk, dg, (float*)op.k, st)));
+  SG_CUDA(cudaStreamSynchronize(st));  // (the copy's source goes)
   const void* kern = elem == 8 ? (const void*)block_kernel<double>(op.TS) : (const void*)block_kernel<float>(op.TS);
   SG_TRY(ensure_smem(kern, op.smem));
   int dev = 0, sms = 0, per_sm = 0;
@@ -574,13 +575,7 @@ int build_block_op(System& s, BlockOp& op, int elem, cudaStream_t st) {
 }
 
 void free_block_op(BlockOp& op) {
-  op.table.release();
-  op.tkind.release();
-  op.err.release();
-  op.k64.release();
-  op.k32.release();
-  op.f64.release();
-  op.f32.release();
+  op.mem.release();
   op.ready = false;
 }
 
@@ -593,8 +588,8 @@ int launch_block_op(const System& s, const BlockOp& op, const T* X, T* Y, T alph
                     test_block_fail()};
   auto kern = block_kernel<T>(op.TS);
   TimeScope ts(s.timer, sizeof(T) == 8 ? K_APPLY_F64 : K_APPLY_LOWP, st);
-  SG_TRY(launch_pdl(kern, dim3(op.grid), dim3((op.nb + 1) * 32), op.smem, st, g, (const int*)op.table.p,
-                    (const int*)op.tkind.p, (const T*)block_store<T>(op), X, F, done, op.err.p));
+  SG_TRY(launch_pdl(kern, dim3(op.grid), dim3((op.nb + 1) * 32), op.smem, st, g, (const int*)op.table,
+                    (const int*)op.tkind, (const T*)op.k, X, F, done, op.err));
   // 16-byte accesses where every row starts on one
   constexpr int kV = 16 / sizeof(T);
   const auto addr = [](const void* p) { return reinterpret_cast<unsigned long long>(p); };

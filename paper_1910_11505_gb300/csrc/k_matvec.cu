@@ -162,7 +162,7 @@ int launch_matvec_f64(const System& s, const double* X, double* Y, double alpha,
                       double beta, cudaStream_t st, const int* done, double* scratch) {
   if (s.block64.ready)
     return launch_block_op<double>(s, s.block64, X, Y, alpha, B, beta,
-                                   scratch ? scratch : s.block64.f64.p, st, done);
+                                   scratch ? scratch : (double*)s.block64.f, st, done);
   if (s.tile64.ready) return launch_tile_op<double>(s, s.tile64, X, Y, alpha, B, beta, st, done);
   return launch_apply<double, double>(s, s.stack.p, s.ent_g.p, X, Y, alpha, B, beta, st, done);
 }
@@ -171,7 +171,7 @@ int launch_matvec_f32(const System& s, const float* X, float* Y, float alpha, co
                       float beta, cudaStream_t st, const int* done, float* scratch) {
   if (s.block32.ready)
     return launch_block_op<float>(s, s.block32, X, Y, alpha, B, beta,
-                                  scratch ? scratch : s.block32.f32.p, st, done);
+                                  scratch ? scratch : (float*)s.block32.f, st, done);
   if (s.tile32.ready && s.prm.precision == SG_MIXED_FP32)
     return launch_tile_op<float>(s, s.tile32, X, Y, alpha, B, beta, st, done);
   if (s.prm.precision == SG_MIXED_BF16)

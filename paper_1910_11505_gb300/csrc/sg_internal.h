@@ -347,9 +347,9 @@ struct BlockOp {
   bool ready = false;
   int elem = 0, TS = 0, nb = 0, rounds = 0, ntile = 0, nval = 0, row_tiles = 0, slots = 0, grid = 0;
   size_t smem = 0, bytes = 0;
-  DBuf<int> table, tkind, err;
-  DBuf<double> k64, f64;
-  DBuf<float> k32, f32;
+  DBuf<unsigned char> mem;  // the tiles k, the products f, the tables and the error word
+  void *k = nullptr, *f = nullptr;
+  int *table = nullptr, *tkind = nullptr, *err = nullptr;
 };
 
 // ------------------------------------------------------------------ per-system state
