@@ -392,11 +392,9 @@ __global__ void __launch_bounds__(1024) color_cta_kernel(int m, int N, int ldN, 
                                                         int fac_per_col, const int* __restrict__ cstart_g,
                                                         const T* __restrict__ cfs,
                                                         T* __restrict__ Rt, T* __restrict__ Z,
-                                                        const int* __restrict__ done,
-                                                        const T* __restrict__ cs, T* __restrict__ corr,
-                                                        int stage) {
-  color_cta_solve<T>(m, N, ldN, P, a0 + (int)blockIdx.x, fac_per_col, cstart_g, cfs, Rt, Z, done, cs,
-                     corr, stage, gridDim.x == 1);
+                                                        const int* __restrict__ done, int stage) {
+  color_cta_solve<T>(m, N, ldN, P, a0 + (int)blockIdx.x, fac_per_col, cstart_g, cfs, Rt, Z, done,
+                     (const T*)nullptr, (T*)nullptr, stage, gridDim.x == 1);
 }
 
 // One step of the Gauss-Seidel sweep: CTA 0 solves block a, the others subtract block a - 1's
@@ -726,11 +724,14 @@ size_t split_smem(int m, int cl) {
 template <typename T, int CL>
 int launch_cluster(System& s, int a0, int ncols, int fac_per_col, const T* lu, T* Rt, T* Z,
                    cudaStream_t st, const int* done, const T* cs, T* corr, bool split) {
-  const size_t smem = split ? split_smem<T>(s.pat.m, CL) : 0;
+  size_t smem = 0;
   ClusterKern<T> kern = color_cluster_kernel<T, CL>;
-  if (smem > 0) {
-    kern = color_split_kernel<T, CL>;
-    SG_TRY(ensure_smem((const void*)kern, smem));
+  if constexpr (sizeof(T) == 4 || CL > 2) {  // (FP64 splits single columns alone, over four CTAs at least)
+    smem = split ? split_smem<T>(s.pat.m, CL) : 0;
+    if (smem > 0) {
+      kern = color_split_kernel<T, CL>;
+      SG_TRY(ensure_smem((const void*)kern, smem));
+    }
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(ncols * CL), 1, 1);
@@ -844,8 +845,8 @@ static bool clusters16(int m, bool in_smem) {
 template <typename T>
 int launch_color_solve(System& s, int a0, int ncols, int fac_per_col, const T* lu, T* Rt, T* Z,
                        cudaStream_t st, const int* done, const T* cs, T* corr) {
-  if (cs != nullptr && (ncols != 1 || corr == nullptr))
-    return fail(SG_ERR_ARG, "four-colour solve: the coupled form takes one column and a buffer");
+  if (cs != nullptr && (ncols != 1 || corr == nullptr || color_one_cta(s)))
+    return fail(SG_ERR_ARG, "four-colour solve: the coupled form takes one column on a cluster, and a buffer");
   const int m = s.pat.m;
   // One CTA with the column in shared memory up to 2048 nodes per colour (two per thread), else a
   // cluster of CTAs, 16 of them only where the device schedules them.  The column in the
@@ -868,7 +869,7 @@ int launch_color_solve(System& s, int a0, int ncols, int fac_per_col, const T* l
     return launch_cluster<T, 2>(s, a0, ncols, fac_per_col, lu, Rt, Z, st, done, cs, corr, split);
   }
   size_t smem = 0;
-  const int stage = color_stage<T>(s, cs != nullptr, smem);
+  const int stage = color_stage<T>(s, false, smem);
   auto kern = color_cta_kernel<T>;
   SG_TRY(ensure_smem((const void*)kern, smem));
   TimeScope ts(s.timer, K_ILU_SOLVE, st);
@@ -883,7 +884,7 @@ int launch_color_solve(System& s, int a0, int ncols, int fac_per_col, const T* l
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   SG_CUDA(cudaLaunchKernelEx(&cfg, kern, m, s.N, s.ldN, s.P, a0, fac_per_col,
-                             (const int*)s.cstart.p, lu, Rt, Z, done, cs, corr, stage));
+                             (const int*)s.cstart.p, lu, Rt, Z, done, stage));
   return check_launch("color_cta");
 }
 
