@@ -63,7 +63,10 @@ size_t smem_optin_max() {
 
 // What the tests of failure paths set on their own thread (sg_test_hook).
 static thread_local int g_test_block_fail = 0;
+static thread_local long long g_test_alloc = 0;
 int test_block_fail() { return g_test_block_fail; }
+// True for the allocation that a test wants to see refused.
+static bool test_alloc_refused() { return g_test_alloc > 0 && --g_test_alloc == 0; }
 
 TimeScope::TimeScope(Timer* t_, int cls_, cudaStream_t st_) : t(t_), cls(cls_), st(st_) {
   if (!t || !t->on) return;
@@ -83,7 +86,7 @@ template <typename T>
 int DBuf<T>::alloc(size_t count) {
   release();
   if (count == 0) count = 1;
-  cudaError_t e = cudaMalloc((void**)&p, sizeof(T) * count);
+  cudaError_t e = test_alloc_refused() ? cudaErrorMemoryAllocation : cudaMalloc((void**)&p, sizeof(T) * count);
   if (e != cudaSuccess) {
     p = nullptr;
     cudaGetLastError();
@@ -866,7 +869,7 @@ static void* captured_scratch(sg_handle* h, size_t bytes, cudaGraph_t graph) {
     void* p = nullptr;
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // allows cudaMalloc on this thread
     cudaThreadExchangeStreamCaptureMode(&mode);
-    const cudaError_t e = cudaMalloc(&p, bytes);
+    const cudaError_t e = test_alloc_refused() ? cudaErrorMemoryAllocation : cudaMalloc(&p, bytes);
     cudaThreadExchangeStreamCaptureMode(&mode);
     if (e != cudaSuccess) {
       cudaGetLastError();
@@ -901,7 +904,8 @@ static int matvec_pooled(sg_handle* h, System& s, cudaStream_t st, Run run, Pair
     return f != nullptr ? run((T*)f) : pairs();
   }
   void* p = nullptr;
-  if (cudaMallocFromPoolAsync(&p, sizeof(T) * block_scratch_elems(s), h->pool, st) != cudaSuccess) {
+  if (test_alloc_refused() ||
+      cudaMallocFromPoolAsync(&p, sizeof(T) * block_scratch_elems(s), h->pool, st) != cudaSuccess) {
     cudaGetLastError();  // no memory for another stream's products: the kernel that needs none
     return pairs();
   }
@@ -1484,10 +1488,12 @@ void sg_free(sg_handle* h) {
 }
 
 // For the tests of failure paths; acts on the calling thread alone.  what 0: value 1 has the CTAs of
-// the block-stencil operator start as if a wait had given up, 0 ends that.
+// the block-stencil operator start as if a wait had given up, 0 ends that.  what 1: the value-th
+// device allocation from now on is refused as out of memory (0: none).
 int sg_test_hook(int what, long long value) {
-  if (what != 0) return fail(SG_ERR_ARG, "unknown hook");
-  g_test_block_fail = value != 0;
+  if (what != 0 && what != 1) return fail(SG_ERR_ARG, "unknown hook");
+  if (what == 0) g_test_block_fail = value != 0;
+  else g_test_alloc = value;
   return SG_OK;
 }
 
