@@ -97,7 +97,12 @@ typedef struct {
   int op_ctas;       /* SG_OP_TILE: CTAs per SM the shared memory is planned for, 1 or 2 (0: 1) */
   int ilu_order;     /* ILU(0) node ordering: SG_ILU_NATURAL, or SG_ILU_COLOR4 (colour           */
                      /* (x mod 2) + 2 (y mod 2), colours in turn: every triangular sweep runs   */
-                     /* in 4 fully parallel phases; requires inner_iters = 1)                   */
+                     /* in 4 fully parallel phases; requires inner_iters = 1).  The natural     */
+                     /* order's solves by warps (FP64: 14 to 132 nodes a side; mixed mean-based  */
+                     /* and Jacobi: 14 to 258) keep a copy of the factors, and are taken while   */
+                     /* it needs at most a sixteenth of the device memory and leaves half of it  */
+                     /* free; else, and after a setup that ran out of memory, the level-by-level */
+                     /* solves serve.  They agree to rounding.                                  */
   int coupling_bf16; /* SG_MIXED_FP32 with a field-split Gauss-Seidel sweep (alone or as the    */
                      /* smoother): 1 = the sweep's coupling sum_{b<a} K_ab z_b reads a BF16     */
                      /* copy of the stiffness values (FP32 arithmetic), half the bytes of the   */
@@ -221,8 +226,9 @@ int sg_export(const sg_handle* h, int sys, int what, void* dst, size_t bytes);
 
 /* Which SG operator kernel system ``sys`` runs: info[0..3] for the FP64 operator and info[4..7]
  * for the FP32 one, each {kernel (0 none, 1 pair kernel, 2 row-tiled kernel, 3 block-stencil
- * operator), kappa (3: fields per range), shared memory bytes, chunks (3: ranges)}; ``msg`` (msg_len bytes, may be NULL) receives why a row-tiled operator
- * was not built ("" if it was). */
+ * operator), kappa (3: fields per range), shared memory bytes, chunks (3: ranges)}; ``msg``
+ * (msg_len bytes, may be NULL) receives how they were chosen: the candidates' times where they were
+ * timed, "(cached)" where an earlier setup had, why a form that was asked for could not be built. */
 int sg_op_info(const sg_handle* h, int sys, long long* info, char* msg, int msg_len);
 
 /* For tests, host only (no device work): plan the row-tiled operator of a system with these sizes
