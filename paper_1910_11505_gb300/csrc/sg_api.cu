@@ -859,7 +859,7 @@ static void CUDART_CB release_captured(void* arg) {
 // Null if there is no memory for it.
 static void* captured_scratch(sg_handle* h, size_t bytes, cudaGraph_t graph) {
   CaptureStore& c = *h->captured;
-  std::lock_guard<std::mutex> lock(c.mu);
+  std::unique_lock<std::mutex> lock(c.mu);
   size_t at = c.blocks.size();
   for (size_t i = 0; i < c.blocks.size(); ++i)  // the smallest free one that is large enough
     if (!c.blocks[i].held && c.blocks[i].bytes >= bytes &&
@@ -885,18 +885,23 @@ static void* captured_scratch(sg_handle* h, size_t bytes, cudaGraph_t graph) {
     return nullptr;
   }
   c.blocks[at].held = true;
+  void* const p = c.blocks[at].p;
+  lock.unlock();
   if (cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove) != cudaSuccess) {
-    cudaUserObjectRelease(obj, 1);  // (its end marks the block free)
     cudaGetLastError();
+    cudaUserObjectRelease(obj, 1);  // (its end, which takes the lock, marks the block free)
     return nullptr;
   }
-  return c.blocks[at].p;
+  return p;
 }
 
 template <typename T, typename Run, typename Pairs>
 static int matvec_pooled(sg_handle* h, System& s, cudaStream_t st, Run run, Pairs pairs) {
   cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &status) != cudaSuccess) cudaGetLastError();
+  if (cudaStreamIsCapturing(st, &status) != cudaSuccess) {
+    cudaGetLastError();
+    status = cudaStreamCaptureStatusNone;
+  }
   if (status == cudaStreamCaptureStatusActive) {
     cudaGraph_t graph = nullptr;
     SG_CUDA(cudaStreamGetCaptureInfo(st, &status, nullptr, &graph, nullptr, nullptr, nullptr));
