@@ -37,13 +37,14 @@ def test_rows_of_a_block_more_than_4_gb_apart():
 
 def test_loss_of_equal_squares():
     # every residual is the same value, so that the rounding of a long FP32 sum does not cancel: 124
-    # tiles of 32 squares a thread (4.8e-5 off as one chain of 3968).  A tile's sum is 32 FP32 additions,
-    # everything after it in FP64 but for two roundings: 34 x 2^-24.
+    # tiles of 32 squares a thread (4.8e-5 off as one chain of 3968).  FP32 additions on the way of a
+    # square: 32 in its tile, 2 for the compensated sum of the tiles, 5 in the warp, 4 over the warps;
+    # then two roundings: 45 x 2^-24.
     B, out, dims = 1024, 300_000, (2, 4, 4)
     net = sg.SGNet(*dims, out, max_batch=B, bf16=True, seed=3)
     net.set_basis(torch.zeros(1, out, device="cuda"))  # W3 = 0 (and b3 = 0)
     T = torch.full((B, out), 0.9, device="cuda")
     loss = net.loss_grad(torch.zeros(B, 2, device="cuda"), T)
     want = float(np.float32(0.9)) ** 2
-    assert abs(loss - want) <= 34 * 2.0 ** -24 * want
+    assert abs(loss - want) <= 45 * 2.0 ** -24 * want
     net.close()
